@@ -261,13 +261,14 @@ template <typename T> lgf_status delta_one(lgf_ctx *g, State<T> &S, int j) {
   return with_fft_type<T>(g, [&](auto tag) -> lgf_status {
     using FT = decltype(tag);
     if constexpr (std::is_same<T, float>::value)
-      k_delta_f32<NT><<<dim3(g->nblocks_site, 1, 1), NT, 0, g->stream>>>(
-          cfg_links(S.U, g, j), cfg_packed(S.P, g, j), g->partials + (int64_t)j * 2 * g->nblocks_site, g->ctrl + j,
-          g->L, 0, 0, 0);
+      k_delta_f32<NT><<<dim3(g->grid32.blocks, 1, 1), NT, 0, g->stream>>>(
+          cfg_links(S.U, g, j), cfg_packed(S.P, g, j), g->partials + (int64_t)j * 2 * g->grid32.blocks, g->ctrl + j,
+          g->L, 0, 0, 0, g->grid32.spt);
     else
-      k_delta<T, NT, FT><<<dim3(g->nblocks_site, 1, 1), NT, 0, g->stream>>>(
+      k_delta<T, NT, FT><<<dim3(g->grid64.blocks, 1, 1), NT, 0, g->stream>>>(
           cfg_links(S.U, g, j), reinterpret_cast<FT *>(cfg_packed(S.P, g, j)),
-          g->partials + (int64_t)j * 2 * g->nblocks_site, g->ctrl + j, g->L, 0, 0, 0);
+          g->partials + (int64_t)j * 2 * g->grid64.blocks, g->ctrl + j, g->L, 0, 0, 0,
+          g->grid64.spt);
     CKL();
     return LGF_OK;
   });
@@ -304,9 +305,10 @@ lgf_status enter_residual_one(lgf_ctx *g, int j, double eps, bool narrow) {
   CKL();
   return with_fft_type<double>(g, [&](auto tag) -> lgf_status {
     using FT = decltype(tag);
-    k_delta_residual<NT, FT><<<dim3(g->nblocks_site, 1, 1), NT, 0, g->stream>>>(
+    k_delta_residual<NT, FT><<<dim3(g->grid_resid.blocks, 1, 1), NT, 0, g->stream>>>(
         g->Rres + (int64_t)j * 72 * V, reinterpret_cast<const FT *>(cfg_packed(g->s64.P, g, j)),
-        cfg_packed(g->s32.P, g, j), g->partials + (int64_t)j * 2 * g->nblocks_site, g->ctrl + j, g->L, 0, 0);
+        cfg_packed(g->s32.P, g, j), g->partials + (int64_t)j * 2 * g->grid_resid.blocks, g->ctrl + j, g->L, 0, 0,
+        g->grid_resid.spt);
     CKL();
     return LGF_OK;
   });

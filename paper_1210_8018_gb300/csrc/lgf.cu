@@ -98,6 +98,10 @@ template <typename T> struct State {
 };
 
 }  // namespace
+struct SiteGrid {
+  int blocks = 0, spt = 1;  // blocks per configuration, sites per thread
+};
+
 
 struct lgf_ctx {
   int n[4];
@@ -129,7 +133,7 @@ struct lgf_ctx {
   double *staging2 = nullptr;
   size_t staging2_bytes = 0;
   double *partials = nullptr;
-  int nblocks_site = 0;
+  SiteGrid grid64, grid32, grid_resid;  // the reducing site kernels in double, float and the residual stage
   int64_t partials_blocks = 0;  // (theta, F) pairs per configuration in partials
   Ctrl *ctrl = nullptr;
   Ctrl ctrl_host{};
@@ -539,11 +543,16 @@ template <typename T> lgf_status setup_precision(lgf_ctx *ctx, State<T> &S) {
 
 lgf_status ensure_common(lgf_ctx *ctx) {
   if (!ctx->partials) {
-    ctx->nblocks_site = (int)((ctx->V + NT * kSitesPerThread - 1) / (NT * kSitesPerThread));
-    // one (theta, F) pair per block of the largest reducing grid: the site kernels' nblocks_site, or the
+    TRY(site_grid(ctx, (const void *)k_delta_f32<NT>, &ctx->grid32));
+    TRY(with_fft_type<double>(ctx, [&](auto tag) -> lgf_status {
+      using FT = decltype(tag);
+      TRY(site_grid(ctx, (const void *)k_delta<double, NT, FT>, &ctx->grid64));
+      return site_grid(ctx, (const void *)k_delta_residual<NT, FT>, &ctx->grid_resid);
+    }));
+    // one (theta, F) pair per block of the largest reducing grid: the site kernels' waves, or the
     // t-walking kernels' columns x Nt / 8 blocks (twalk_on)
-    ctx->partials_blocks = std::max<int64_t>(
-        std::max(ctx->nblocks_site, 1), (ctx->L.stride[3] + NT - 1) / NT * std::max(ctx->n[3] / 8, 1));
+    ctx->partials_blocks = std::max<int64_t>(std::max({ctx->grid64.blocks, ctx->grid32.blocks, ctx->grid_resid.blocks}),
+                                             (ctx->L.stride[3] + NT - 1) / NT * std::max(ctx->n[3] / 8, 1));
     CK(cudaMalloc(&ctx->partials, sizeof(double) * 2 * (size_t)ctx->partials_blocks * ctx->nb));
     CK(cudaMalloc(&ctx->ctrl, sizeof(Ctrl) * ctx->nb));
     CK(cudaMemset(ctx->ctrl, 0, sizeof(Ctrl) * ctx->nb));
@@ -592,6 +601,30 @@ lgf_status input_ptr(lgf_ctx *ctx, const double *p, size_t bytes, double **buf, 
   TRY(ensure_staging(ctx, buf, have, bytes));
   CK(cudaMemcpyAsync(*buf, p, bytes, cudaMemcpyHostToDevice, ctx->stream));
   *out = *buf;
+// Sites per thread (1 to 4) and blocks of a reducing site kernel, per configuration: the fewest rounds of sites
+// over the waves of blocks, with a block's reduction and start counted as half a round. Four everywhere left
+// most of the GPU idle on small lattices (float Delta at 8^4, 4 blocks: 20.4 us, now 13.3; double at 18x12x10x15:
+// 48 -> 21) and a nearly empty last wave on others (double at 24^3x48: 177 -> 158 us; float at 32^4: 71 -> 67).
+// Without the count for the block, one site per thread would be taken where four are faster (residual Delta at
+// 32^4: 104 against 88 us). One wave of blocks that step through the whole lattice was slower in double (64^4:
+// 5.7 against 3.4 ms).
+lgf_status site_grid(lgf_ctx *ctx, const void *kernel, SiteGrid *g) {
+  int per_sm = 0;
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, 0));
+  const int64_t wave = (int64_t)std::max(per_sm, 1) * ctx->num_sms, chunks = (ctx->V + NT - 1) / NT;
+  double best = 0;
+  for (int spt = 4; spt >= 1; --spt) {
+    const int64_t blocks = (chunks + spt - 1) / spt;
+    const double cost = (double)((blocks * ctx->nb + wave - 1) / wave) * (spt + 0.5);
+    if (best == 0 || cost < best) {
+      best = cost;
+      g->spt = spt;
+      g->blocks = (int)blocks;
+    }
+  }
+  return LGF_OK;
+}
+
   return LGF_OK;
 }
 
@@ -631,19 +664,18 @@ template <typename T> lgf_status launch_delta(lgf_ctx *ctx, State<T> &S, int cou
   TRY(timed_begin(ctx, kid<T>(KID_DELTA)));
   TRY(with_fft_type<T>(ctx, [&](auto tag) -> lgf_status {
     using FT = decltype(tag);
-    const dim3 grid(ctx->nblocks_site, 1, ctx->nb);
     FT *P = reinterpret_cast<FT *>(S.P);
     if constexpr (std::is_same<T, float>::value) {
       if (twalk_on(ctx))
         k_delta_f32_tw<NT, kTwalkSlices><<<twalk_grid(ctx), NT, 0, ctx->stream>>>(
             S.U, P, ctx->partials, ctx->ctrl, ctx->L, counts_update, check_active, kid<T>(KID_DELTA));
       else
-        k_delta_f32<NT><<<grid, NT, 0, ctx->stream>>>(S.U, P, ctx->partials, ctx->ctrl, ctx->L, counts_update,
-                                                      check_active, kid<T>(KID_DELTA));
+        k_delta_f32<NT><<<dim3(ctx->grid32.blocks, 1, ctx->nb), NT, 0, ctx->stream>>>(S.U, P, ctx->partials, ctx->ctrl, ctx->L, counts_update,
+                                                      check_active, kid<T>(KID_DELTA), ctx->grid32.spt);
     }
     else
-      k_delta<T, NT, FT><<<grid, NT, 0, ctx->stream>>>(S.U, P, ctx->partials, ctx->ctrl, ctx->L, counts_update,
-                                                       check_active, kid<T>(KID_DELTA));
+      k_delta<T, NT, FT><<<dim3(ctx->grid64.blocks, 1, ctx->nb), NT, 0, ctx->stream>>>(S.U, P, ctx->partials, ctx->ctrl, ctx->L, counts_update,
+                                                       check_active, kid<T>(KID_DELTA), ctx->grid64.spt);
     CKL();
     return LGF_OK;
   }));
@@ -729,8 +761,9 @@ template <typename T> lgf_status launch_iteration(lgf_ctx *ctx, State<T> &S, dou
 // packed in float, float FFT passes, g formed in double from the float Delta-tilde, double update.
 lgf_status launch_delta_d2f(lgf_ctx *ctx, int counts_update, int check_active) {
   TRY(timed_begin(ctx, kid<double>(KID_DELTA)));
-  k_delta<double, NT, float><<<dim3(ctx->nblocks_site, 1, ctx->nb), NT, 0, ctx->stream>>>(
-      ctx->s64.U, ctx->s32.P, ctx->partials, ctx->ctrl, ctx->L, counts_update, check_active, kid<double>(KID_DELTA));
+  k_delta<double, NT, float><<<dim3(ctx->grid64.blocks, 1, ctx->nb), NT, 0, ctx->stream>>>(
+      ctx->s64.U, ctx->s32.P, ctx->partials, ctx->ctrl, ctx->L, counts_update, check_active, kid<double>(KID_DELTA),
+      ctx->grid64.spt);
   CKL();
   return timed_end(ctx);
 }
@@ -829,9 +862,9 @@ lgf_status launch_delta_residual(lgf_ctx *ctx, int counts_update) {
           ctx->Rres, reinterpret_cast<const FT *>(ctx->s64.P), ctx->s32.P, ctx->partials, ctx->ctrl, ctx->L,
           counts_update, kid<float>(KID_DELTA_RESIDUAL));
     else
-      k_delta_residual<NT, FT><<<dim3(ctx->nblocks_site, 1, ctx->nb), NT, 0, ctx->stream>>>(
+      k_delta_residual<NT, FT><<<dim3(ctx->grid_resid.blocks, 1, ctx->nb), NT, 0, ctx->stream>>>(
           ctx->Rres, reinterpret_cast<const FT *>(ctx->s64.P), ctx->s32.P, ctx->partials, ctx->ctrl, ctx->L,
-          counts_update, kid<float>(KID_DELTA_RESIDUAL));
+          counts_update, kid<float>(KID_DELTA_RESIDUAL), ctx->grid_resid.spt);
     CKL();
     return LGF_OK;
   }));
@@ -1440,7 +1473,8 @@ lgf_status lgf_measure(lgf_ctx *ctx, const double *links, double *theta, double 
   TRY(launch_delta<double>(ctx, ctx->s64, 0, 0));
   if (plaq) {
     // stream-ordered after the Delta reduction, which leaves the last-block counter at zero
-    k_plaquette<double, NT><<<ctx->nblocks_site, NT, 0, ctx->stream>>>(ctx->s64.U, ctx->partials, ctx->ctrl, ctx->L);
+    k_plaquette<double, NT><<<ctx->grid64.blocks, NT, 0, ctx->stream>>>(ctx->s64.U, ctx->partials, ctx->ctrl, ctx->L,
+                                                                   ctx->grid64.spt);
     CKL();
   }
   TRY(read_ctrl(ctx));
@@ -1480,8 +1514,8 @@ template <typename T> static lgf_status step_delta(lgf_ctx *ctx, State<T> &S, co
   TRY(write_ctrl(ctx));
   if constexpr (std::is_same<T, double>::value) {
     // the caller gets Delta in full FP64: pack it as double, not as the type of the double path's FFT
-    k_delta<double, NT, double><<<dim3(ctx->nblocks_site, 1, 1), NT, 0, ctx->stream>>>(
-        S.U, S.P, ctx->partials, ctx->ctrl, ctx->L, 0, 0, kid<T>(KID_DELTA));
+    k_delta<double, NT, double><<<dim3(ctx->grid64.blocks, 1, 1), NT, 0, ctx->stream>>>(
+        S.U, S.P, ctx->partials, ctx->ctrl, ctx->L, 0, 0, kid<T>(KID_DELTA), ctx->grid64.spt);
     CKL();
     k_unpack_antiherm<double><<<grid1(V, NT), NT, 0, ctx->stream>>>(S.P, dst, V);
     CKL();
@@ -1693,8 +1727,8 @@ extern "C" lgf_status lgf_functional(lgf_ctx *ctx, const double *links, const do
   const int64_t V = ctx->V;
   memset(&ctx->ctrl_host, 0, sizeof(Ctrl));
   TRY(write_ctrl(ctx));
-  k_functional_g<NT><<<ctx->nblocks_site, NT, 0, ctx->stream>>>(ctx->s64.U, ctx->s64.G, ctx->partials, ctx->ctrl,
-                                                                ctx->L);
+  k_functional_g<NT><<<ctx->grid64.blocks, NT, 0, ctx->stream>>>(ctx->s64.U, ctx->s64.G, ctx->partials, ctx->ctrl,
+                                                                ctx->L, ctx->grid64.spt);
   CKL();
   if (g_out) {
     double *gdev = nullptr;

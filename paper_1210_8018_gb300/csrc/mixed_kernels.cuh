@@ -347,7 +347,7 @@ template <typename T> __device__ __forceinline__ void load9(const T *plane, int6
 template <int NT, typename PT>
 __global__ void __launch_bounds__(NT, 4) k_delta_residual(const float *__restrict__ R, const PT *__restrict__ Ph,
                                                       float *__restrict__ P, double *partials, Ctrl *ctrl, Lattice L,
-                                                      int counts_update, int tkid) {
+                                                      int counts_update, int tkid, int spt) {
   const int64_t V = L.V;
   {
     const int cfg = blockIdx.z;
@@ -361,8 +361,8 @@ __global__ void __launch_bounds__(NT, 4) k_delta_residual(const float *__restric
   count_run(ctrl, tkid);
   double th = 0.0, f = 0.0;
 #pragma unroll 1
-  for (int k = 0; k < kSitesPerThread; ++k) {
-    const int64_t s = ((int64_t)blockIdx.x * kSitesPerThread + k) * NT + threadIdx.x;
+  for (int k = 0; k < spt; ++k) {
+    const int64_t s = ((int64_t)blockIdx.x * spt + k) * NT + threadIdx.x;
     if (s >= V) break;
     int c[4];
     site_coords(L, s, c);

@@ -186,14 +186,13 @@ __device__ __forceinline__ void reduce_and_finalize(double th, double f, double 
 
 // ---------------------------------------------------------------------------------------------
 // a1/a2: Delta(x) = sum_nu [U_nu(x-nu) - U_nu(x) - h.c. - trace] (Eqs. 3, 5), theta and F partials.
-// Each thread handles kSitesPerThread sites (consecutive threads take consecutive sites). Only the
+// Each thread handles spt sites one after another (consecutive threads take consecutive sites; SiteGrid
+// chooses spt). Only the
 // nine real combinations that the anti-Hermitian traceless part needs are accumulated:
 //   (B_01 - conj B_10), (B_02 - conj B_20), (B_12 - conj B_21) and Im B_00, Im B_11, Im B_22,
 // with B = sum_nu [U_nu(x - nu) - U_nu(x)]. The per-site theta and F are formed in the kernel's
 // precision and accumulated in double; the warp, block and global sums are double.
 // ---------------------------------------------------------------------------------------------
-constexpr int kSitesPerThread = 4;
-
 template <typename T> __device__ __forceinline__ void accumulate_link(const m3<T> &u, T sign, T acc[9]) {
   acc[0] = fma(sign, u.e[1].r - u.e[3].r, acc[0]);
   acc[1] = fma(sign, u.e[1].i + u.e[3].i, acc[1]);
@@ -246,7 +245,7 @@ __device__ __forceinline__ double widen_exact(double v) { return v; }
 // PT is the type of the packed output (T, or float when a double stage feeds a float FFT).
 template <typename T, int NT, typename PT = T>
 __device__ __forceinline__ void delta_body(const T *__restrict__ U, PT *__restrict__ P, double *partials, Ctrl *ctrl,
-                                           Lattice L, int counts_update, int check_active, int tkid) {
+                                           Lattice L, int counts_update, int check_active, int tkid, int spt) {
   const int64_t V = L.V;
   {
     const int cfg = blockIdx.z;
@@ -260,8 +259,8 @@ __device__ __forceinline__ void delta_body(const T *__restrict__ U, PT *__restri
   double th = 0.0, f = 0.0;
   if constexpr (std::is_same<T, double>::value) {
 #pragma unroll 1
-    for (int k = 0; k < kSitesPerThread; ++k) {
-      const int64_t s = ((int64_t)blockIdx.x * kSitesPerThread + k) * NT + threadIdx.x;
+    for (int k = 0; k < spt; ++k) {
+      const int64_t s = ((int64_t)blockIdx.x * spt + k) * NT + threadIdx.x;
       if (s >= V) break;
       int c[4];
       site_coords(L, s, c);
@@ -301,8 +300,8 @@ __device__ __forceinline__ void delta_body(const T *__restrict__ U, PT *__restri
     }
   } else {
 #pragma unroll 1
-    for (int k = 0; k < kSitesPerThread; ++k) {
-      const int64_t s = ((int64_t)blockIdx.x * kSitesPerThread + k) * NT + threadIdx.x;
+    for (int k = 0; k < spt; ++k) {
+      const int64_t s = ((int64_t)blockIdx.x * spt + k) * NT + threadIdx.x;
       if (s >= V) break;
       int c[4];
       site_coords(L, s, c);
@@ -339,8 +338,8 @@ __device__ __forceinline__ void delta_body(const T *__restrict__ U, PT *__restri
 
 template <typename T, int NT, typename PT = T>
 __global__ void __launch_bounds__(NT) k_delta(const T *__restrict__ U, PT *__restrict__ P, double *partials, Ctrl *ctrl,
-                                             Lattice L, int counts_update, int check_active, int tkid) {
-  delta_body<T, NT, PT>(U, P, partials, ctrl, L, counts_update, check_active, tkid);
+                                             Lattice L, int counts_update, int check_active, int tkid, int spt) {
+  delta_body<T, NT, PT>(U, P, partials, ctrl, L, counts_update, check_active, tkid, spt);
 }
 // The float stage's Delta with five resident blocks per SM asked of the compiler (48 registers, 40 warps in
 // flight instead of 32): the kernel waits on its link loads, and more warps hide that latency (measured at
@@ -348,8 +347,8 @@ __global__ void __launch_bounds__(NT) k_delta(const T *__restrict__ U, PT *__res
 template <int NT>
 __global__ void __launch_bounds__(NT, 5) k_delta_f32(const float *__restrict__ U, float *__restrict__ P,
                                                      double *partials, Ctrl *ctrl, Lattice L, int counts_update,
-                                                     int check_active, int tkid) {
-  delta_body<float, NT, float>(U, P, partials, ctrl, L, counts_update, check_active, tkid);
+                                                     int check_active, int tkid, int spt) {
+  delta_body<float, NT, float>(U, P, partials, ctrl, L, counts_update, check_active, tkid, spt);
 }
 
 // The float Delta walking along t: thread (x, y, z) takes the TCH t-slices of chunk blockIdx.y, and the
@@ -956,11 +955,12 @@ template <typename PT> __global__ void k_unpack_coeffs(const PT *__restrict__ P,
 
 // Average plaquette partials: (1/3) Re Tr U_mu(x) U_nu(x+mu) U_mu^+(x+nu) U_nu^+(x) over mu < nu.
 template <typename T, int NT>
-__global__ void __launch_bounds__(NT) k_plaquette(const T *__restrict__ U, double *partials, Ctrl *ctrl, Lattice L) {
+__global__ void __launch_bounds__(NT) k_plaquette(const T *__restrict__ U, double *partials, Ctrl *ctrl, Lattice L,
+                                                 int spt) {
   const int64_t V = L.V;
   double acc = 0.0;
-  for (int k = 0; k < kSitesPerThread; ++k) {
-    const int64_t s = ((int64_t)blockIdx.x * kSitesPerThread + k) * NT + threadIdx.x;
+  for (int k = 0; k < spt; ++k) {
+    const int64_t s = ((int64_t)blockIdx.x * spt + k) * NT + threadIdx.x;
     if (s >= V) break;
     int c[4];
     site_coords(L, s, c);
