@@ -92,7 +92,8 @@ template <typename T> lgf_status apply_fft_choice(lgf_ctx *ctx, State<T> &S, boo
   ctx->generic_fft = generic;
   ctx->fixed_cols[sizeof(T) == 8 ? 0 : 1] = C;
   plan_passes<T>(ctx, S);
-  return opt_in_smem<T>(ctx, S);
+  TRY(opt_in_smem<T>(ctx, S));
+  return ensure_weights<T>(ctx, S);
 }
 
 // Time the filter passes of the current plan (ms per application, median of 5 after 2 warm-ups).

@@ -1,8 +1,8 @@
 // fft.cuh -- hand-written batched 4D FFT with the Fourier-acceleration filter of Algorithm 1.
 //
 // Each packed Delta field (4 per site, see site_kernels.cuh) is transformed by a sequence of
-// "passes". A pass stages a tile of the field in shared memory -- the full extent of one or two
-// lattice axes times a run of C elements that are contiguous in memory -- transforms the tile along
+// "passes". A pass stages a tile of the field in shared memory -- whole xy planes or lattice rows, or the
+// full extent of one or two lattice axes times C neighbouring columns -- transforms the tile along
 // those axes and writes it back. The forward transform is an in-place mixed-radix decimation-in-
 // frequency FFT, which leaves the spectrum in digit-reversed order; the filter reads the frequency of
 // each position from tables, and the inverse runs the exact inverse stages (decimation in time) in
@@ -27,19 +27,41 @@ struct AxisFFT {
   int R[kMaxStages];      // radix of each DIF stage, in forward order
 };
 
-// One pass: a tile of extents d[0] (fastest in shared memory) x d[1] x d[2]; tile element
-// (i0, i1, i2) lives at global complex index base(b) + i0*g[0] + i1*g[1] + i2*g[2] of a field, with
-// base(b) = (b % nb1)*B1 + (b / nb1)*B2 for block b. The pass transforms along nax tile dimensions.
+// n / d for n d < 2^32 by one high multiplication (m = ceil(2^32 / d); d = 1 has m = 0): the lengths of a
+// general lattice are known only at run time, and the hardware has no integer division.
+struct FastDiv {
+  unsigned d, m;
+};
+inline FastDiv fast_div(unsigned d) {
+  return FastDiv{d, d == 1 ? 0u : (unsigned)((((unsigned long long)1 << 32) + d - 1) / d)};
+}
+__device__ __forceinline__ unsigned div_by(unsigned n, FastDiv f) { return f.m ? __umulhi(n, f.m) : n; }
+
+// The transform of a tile along one of its axes: npen pencils of N elements `estride` apart, pencil p
+// starting at (p / A) B + (p % A) S.
+struct AxisPhase {
+  int mu;                    // lattice axis
+  int nst, R[kMaxStages];    // radix of each DIF stage, in forward order
+  FastDiv M[kMaxStages];     // block length of each stage over its radix
+  int N, npen, A, B, S, estride;
+  FastDiv dpen, dA;
+};
+
+// One pass: tiles of one packed field are staged in shared memory and transformed along one or two axes.
+//   columns (rowform 0): C neighbouring columns by `rows` rows, element (row, c) of the tile at
+//     base(q) + row rstride with q = tile C + c, base(q) = (q % nin) + (q / nin) ostride; ncol columns;
+//   rows (rowform 1): `rows` consecutive lattice rows of nx elements (whole xy planes, or rows alone).
 struct PassDesc {
-  int d[3];
-  int64_t g[3];
-  int nb1;
-  int64_t B1, B2;
+  int rowform;
+  int rows, C, logC, pitch;
+  unsigned ncol, nin;
+  int64_t ostride, rstride;
+  unsigned nrow;
+  FastDiv dnx;
   int nax;
-  int ax_dim[2];   // tile dimension of each transformed axis
-  int ax_mu[2];    // lattice axis (0..3) of each
-  int mode;        // 0 forward, 1 inverse, 2 forward + filter + inverse
-  int nblocks;     // blocks per field
+  AxisPhase ph[2];
+  int mode;     // 0 forward, 1 inverse, 2 forward + filter + inverse
+  int nblocks;  // tiles per field
 };
 
 struct FFTTables {
@@ -47,6 +69,7 @@ struct FFTTables {
   const void *tw[4];        // per lattice axis: N complex twiddles w_N^j (T)
   const double *p2part[4];  // per lattice axis: 4 sin^2(pi k(pos)/N) for the frequency at position pos
   double wscale;            // p^2_max / V
+  const void *weights;      // w of every site in the transform's type (the general passes), or null
   int n[4];
 };
 
@@ -145,24 +168,24 @@ template <typename T, int R, bool INV> __device__ __forceinline__ void dft(cx<T>
   else dft8<T, INV>(v);
 }
 
-// One stage over every pencil of the tile along tile dimension a (element stride st, length N).
-// Work item w -> (ilo, butterfly beta, ihi); the contiguous index ilo varies fastest so that
-// consecutive threads touch consecutive shared-memory words.
+// One stage over every pencil of the tile. Work item w -> (pencil p, butterfly beta) with the pencil
+// varying fastest, so that consecutive threads touch consecutive words (or rows of odd pitch) of the tile.
 template <typename T, int R, bool INV>
-__device__ __forceinline__ void fft_stage(cx<T> *tile, const cx<T> *tw, int N, int L, int st, int total_items) {
-  const int M = L / R;
-  const int nb = N / R;       // butterflies per pencil
-  const int twstep = N / L;   // w_L^e = w_N^(e N/L)
-  for (int w = threadIdx.x; w < total_items; w += blockDim.x) {
-    const int ilo = w % st;
-    const int rest = w / st;
-    const int beta = rest % nb;
-    const int ihi = rest / nb;
-    const int blk = beta / M, j = beta - blk * M;
-    const int base = ilo + st * (N * ihi + blk * L + j);
+__device__ __forceinline__ void fft_stage(cx<T> *tile, const cx<T> *tw, const AxisPhase &ph, FastDiv dM) {
+  const unsigned M = dM.d;
+  const unsigned L = M * R;
+  const unsigned twstep = ph.N / L;  // w_L^e = w_N^(e N/L)
+  const unsigned items = ph.npen * (ph.N / R);
+  const int step = M * ph.estride;
+#pragma unroll 1
+  for (unsigned w = threadIdx.x; w < items; w += blockDim.x) {
+    const unsigned beta = div_by(w, ph.dpen), p = w - beta * ph.npen;
+    const unsigned a = div_by(p, ph.dA);
+    const unsigned blk = div_by(beta, dM), j = beta - blk * M;
+    cx<T> *q = tile + (int)(a * ph.B + (p - a * ph.A) * ph.S + (blk * L + j) * ph.estride);
     cx<T> v[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = tile[base + st * M * r];
+    for (int r = 0; r < R; ++r) v[r] = q[r * step];
     // (a stage with M = 1 has j = 0 and unit twiddles: no multiplications; M is uniform per stage)
     if constexpr (!INV) {
       dft<T, R, false>(v);
@@ -178,113 +201,126 @@ __device__ __forceinline__ void fft_stage(cx<T> *tile, const cx<T> *tw, int N, i
       dft<T, R, true>(v);
     }
 #pragma unroll
-    for (int r = 0; r < R; ++r) tile[base + st * M * r] = v[r];
+    for (int r = 0; r < R; ++r) q[r * step] = v[r];
   }
 }
 
 template <typename T, bool INV>
-__device__ __forceinline__ void fft_stage_any(int R, cx<T> *tile, const cx<T> *tw, int N, int L, int st, int items) {
+__device__ __forceinline__ void fft_stage_any(int R, cx<T> *tile, const cx<T> *tw, const AxisPhase &ph, FastDiv dM) {
   switch (R) {
-    case 2: fft_stage<T, 2, INV>(tile, tw, N, L, st, items); break;
-    case 3: fft_stage<T, 3, INV>(tile, tw, N, L, st, items); break;
-    case 4: fft_stage<T, 4, INV>(tile, tw, N, L, st, items); break;
-    case 5: fft_stage<T, 5, INV>(tile, tw, N, L, st, items); break;
-    default: fft_stage<T, 8, INV>(tile, tw, N, L, st, items); break;
+    case 2: fft_stage<T, 2, INV>(tile, tw, ph, dM); break;
+    case 3: fft_stage<T, 3, INV>(tile, tw, ph, dM); break;
+    case 4: fft_stage<T, 4, INV>(tile, tw, ph, dM); break;
+    case 5: fft_stage<T, 5, INV>(tile, tw, ph, dM); break;
+    default: fft_stage<T, 8, INV>(tile, tw, ph, dM); break;
   }
 }
 
-// Full forward (DIF, digit-reversed output) or inverse (DIT, natural output) transform along a tile dim.
+// Full forward (DIF, digit-reversed output) or inverse (DIT, natural output) transform along one axis.
 template <typename T, bool INV>
-__device__ __forceinline__ void fft_axis(cx<T> *tile, const cx<T> *tw, const AxisFFT &ax, int st, int tile_elems) {
-  const int N = ax.N;
-  if (N == 1) return;
-  if (!INV) {
-    int L = N;
-    for (int k = 0; k < ax.nst; ++k) {
-      const int R = ax.R[k];
-      fft_stage_any<T, false>(R, tile, tw, N, L, st, tile_elems / R);
-      __syncthreads();
-      L /= R;
-    }
-  } else {
-    int L = 1;
-    for (int k = ax.nst - 1; k >= 0; --k) {
-      const int R = ax.R[k];
-      L *= R;
-      fft_stage_any<T, true>(R, tile, tw, N, L, st, tile_elems / R);
-      __syncthreads();
-    }
+__device__ __forceinline__ void fft_axis(cx<T> *tile, const cx<T> *tw, const AxisPhase &ph) {
+#pragma unroll 1
+  for (int i = 0; i < ph.nst; ++i) {
+    const int k = INV ? ph.nst - 1 - i : i;
+    fft_stage_any<T, INV>(ph.R[k], tile, tw, ph, ph.M[k]);
+    __syncthreads();
   }
+}
+
+// Filter weight of every site for the general passes, w = p^2_max / (V p^2), 0 at p = 0: in double, rounded
+// once. Kept as a table because p^2 at a (digit-reversed) position and its quotient cost three 64-bit
+// divisions and one FP64 division per element when they are formed inside the pass.
+template <typename T>
+__global__ void k_filter_weights(T *__restrict__ W, int64_t V, FFTTables tb) {
+  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= V) return;
+  unsigned r = (unsigned)s;
+  const unsigned px = r % (unsigned)tb.n[0];
+  r /= (unsigned)tb.n[0];
+  const unsigned py = r % (unsigned)tb.n[1];
+  r /= (unsigned)tb.n[1];
+  const unsigned pz = r % (unsigned)tb.n[2], pt = r / (unsigned)tb.n[2];
+  const double p2 = __ldg(tb.p2part[0] + px) + __ldg(tb.p2part[1] + py) + __ldg(tb.p2part[2] + pz) +
+                    __ldg(tb.p2part[3] + pt);
+  W[s] = p2 == 0.0 ? kconst<T>(0.0) : convert<T>(tb.wscale / p2);
 }
 
 // The pass kernel. blockIdx.x: tile, blockIdx.y: packed field. Shared memory: the tile, then the
 // twiddle tables of the transformed axes.
+// The fields of the lattices that come here mostly fit the L2, and what bounds a pass is issue and the latency
+// of its phases. Index arithmetic is one high multiplication per division, a thread of a column tile keeps its
+// column, and the filter's weight is one load. Measured per launch against passes with run-time division and
+// weights formed in place (ncu: 3-4% of DRAM, 25-58% of the SM, the FP64 pipe 40% busy with the weights):
+// 30x20x24x36 float, z and t with the filter 166 -> 39 us, xy 60 -> 24 us; 18x12x10x15 double-float, 66 -> 19 us
+// and 19 -> 11 us. The operations and their order are those of the earlier passes: the same bits.
 template <typename T>
-__global__ void __launch_bounds__(512) k_fft_pass(T *__restrict__ data, int64_t V, PassDesc pd, FFTTables tb,
-                                                 const Ctrl *ctrl, int check_active, int tkid) {
+__global__ void __launch_bounds__(512) k_fft_pass(T *__restrict__ data, int64_t V, const __grid_constant__ PassDesc pd,
+                                                 const __grid_constant__ FFTTables tb, const Ctrl *ctrl,
+                                                 int check_active, int tkid) {
   data += (int64_t)blockIdx.z * 4 * V * 2;
   ctrl += blockIdx.z;
   if (!should_run<T>(ctrl, check_active)) return;
   count_run(ctrl, tkid);
+  using V2 = typename vec2<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T> *tile = reinterpret_cast<cx<T> *>(smem_raw);
-  const int d0 = pd.d[0], d1 = pd.d[1], d2 = pd.d[2];
-  const int nel = d0 * d1 * d2;
-  cx<T> *twb = tile + nel;
-  // twiddles of the transformed axes
-  int twoff[2] = {0, 0};
-  {
-    int off = 0;
-    for (int a = 0; a < pd.nax; ++a) {
-      const int mu = pd.ax_mu[a];
-      const int N = tb.ax[mu].N;
-      const cx<T> *src = reinterpret_cast<const cx<T> *>(tb.tw[mu]);
-      for (int k = threadIdx.x; k < N; k += blockDim.x) twb[off + k] = src[k];
-      twoff[a] = off;
-      off += N;
-    }
+  cx<T> *twb = tile + pd.rows * pd.pitch;
+  const cx<T> *tw[2] = {twb, twb + pd.ph[0].N};
+  for (int a = 0; a < pd.nax; ++a) {
+    const cx<T> *src = reinterpret_cast<const cx<T> *>(tb.tw[pd.ph[a].mu]);
+    cx<T> *dst = twb + (a ? pd.ph[0].N : 0);
+    for (int k = threadIdx.x; k < pd.ph[a].N; k += blockDim.x) dst[k] = src[k];
   }
-  const int b = blockIdx.x;
-  const int64_t base = (int64_t)(b % pd.nb1) * pd.B1 + (int64_t)(b / pd.nb1) * pd.B2;
-  T *field = data + (int64_t)blockIdx.y * V * 2;
-  // load the tile (consecutive threads read consecutive i0: runs of d0 contiguous elements)
-  for (int e = threadIdx.x; e < nel; e += blockDim.x) {
-    const int i0 = e % d0, r = e / d0, i1 = r % d1, i2 = r / d1;
-    tile[e] = ld(field, base + i0 * pd.g[0] + i1 * pd.g[1] + i2 * pd.g[2]);
+  V2 *field = reinterpret_cast<V2 *>(data + (int64_t)blockIdx.y * V * 2);
+  // this thread's column (column form), or the tile's run of elements (row form)
+  const int c = threadIdx.x & (pd.C - 1), row0 = threadIdx.x >> pd.logC, rstep = blockDim.x >> pd.logC;
+  int64_t base = 0;
+  int rows = pd.rows, nel = 0;
+  if (pd.rowform) {
+    const unsigned r0 = blockIdx.x * (unsigned)pd.rows;
+    nel = (int)min((unsigned)pd.rows, pd.nrow - r0) * (int)pd.dnx.d;
+    base = (int64_t)r0 * pd.dnx.d;
+    for (int e = threadIdx.x; e < pd.rows * (int)pd.dnx.d; e += blockDim.x) {
+      const unsigned r = div_by(e, pd.dnx), x = e - r * pd.dnx.d;
+      V2 v = {};
+      if (e < nel) v = __ldg(field + base + e);
+      tile[r * pd.pitch + x] = from_vec<T>(v);
+    }
+  } else {
+    const unsigned q = blockIdx.x * (unsigned)pd.C + c;
+    if (q >= pd.ncol) rows = 0;  // columns beyond the last: zeros in the tile, nothing stored
+    base = (int64_t)(q % pd.nin) + (int64_t)(q / pd.nin) * pd.ostride;
+#pragma unroll 4
+    for (int r = row0; r < pd.rows; r += rstep) {
+      V2 v = {};
+      if (r < rows) v = __ldg(field + base + r * pd.rstride);
+      tile[r * pd.pitch + c] = from_vec<T>(v);
+    }
   }
   __syncthreads();
-  const int tstride[3] = {1, d0, d0 * d1};
-  if (pd.mode == 0 || pd.mode == 2) {
-    for (int a = 0; a < pd.nax; ++a)
-      fft_axis<T, false>(tile, twb + twoff[a], tb.ax[pd.ax_mu[a]], tstride[pd.ax_dim[a]], nel);
-  } else {
-    for (int a = pd.nax - 1; a >= 0; --a)
-      fft_axis<T, true>(tile, twb + twoff[a], tb.ax[pd.ax_mu[a]], tstride[pd.ax_dim[a]], nel);
+  if (pd.mode != 1) {
+    for (int a = 0; a < pd.nax; ++a) fft_axis<T, false>(tile, tw[a], pd.ph[a]);
   }
   if (pd.mode == 2) {
-    // filter: w = p2max / (V p2(k)) at every position; the site index gives the (digit-reversed)
-    // position along each lattice axis.
-    for (int e = threadIdx.x; e < nel; e += blockDim.x) {
-      const int i0 = e % d0, r = e / d0, i1 = r % d1, i2 = r / d1;
-      int64_t s = base + i0 * pd.g[0] + i1 * pd.g[1] + i2 * pd.g[2];
-      const int px = (int)(s % tb.n[0]);
-      s /= tb.n[0];
-      const int py = (int)(s % tb.n[1]);
-      s /= tb.n[1];
-      const int pz = (int)(s % tb.n[2]);
-      const int pt = (int)(s / tb.n[2]);
-      const double p2 = __ldg(tb.p2part[0] + px) + __ldg(tb.p2part[1] + py) + __ldg(tb.p2part[2] + pz) +
-                        __ldg(tb.p2part[3] + pt);
-      const T w = p2 == 0.0 ? kconst<T>(0.0) : convert<T>(tb.wscale / p2);
-      tile[e] = scale(tile[e], w);
+    // only column passes end with the filter; the weight is read at the site's own index
+    const T *W = reinterpret_cast<const T *>(tb.weights);
+#pragma unroll 4
+    for (int r = row0; r < rows; r += rstep) {
+      cx<T> &v = tile[r * pd.pitch + c];
+      v = scale(v, W[base + r * pd.rstride]);
     }
     __syncthreads();
-    for (int a = pd.nax - 1; a >= 0; --a)
-      fft_axis<T, true>(tile, twb + twoff[a], tb.ax[pd.ax_mu[a]], tstride[pd.ax_dim[a]], nel);
   }
-  for (int e = threadIdx.x; e < nel; e += blockDim.x) {
-    const int i0 = e % d0, r = e / d0, i1 = r % d1, i2 = r / d1;
-    st(field, base + i0 * pd.g[0] + i1 * pd.g[1] + i2 * pd.g[2], tile[e]);
+  if (pd.mode != 0) {
+    for (int a = pd.nax - 1; a >= 0; --a) fft_axis<T, true>(tile, tw[a], pd.ph[a]);
+  }
+  if (pd.rowform) {
+    for (int e = threadIdx.x; e < nel; e += blockDim.x) {
+      const unsigned r = div_by(e, pd.dnx), x = e - r * pd.dnx.d;
+      field[base + e] = to_vec<T>(tile[r * pd.pitch + x]);
+    }
+  } else {
+    for (int r = row0; r < rows; r += rstep) field[base + r * pd.rstride] = to_vec<T>(tile[r * pd.pitch + c]);
   }
 }
 

@@ -93,15 +93,16 @@ template <typename T> struct State {
   T *G = nullptr;  // g, 9 planes
   float *A = nullptr;  // double path: a = g - 1 in double-float, 9 planes of float4
   void *tw[4] = {nullptr, nullptr, nullptr, nullptr};
+  void *weights = nullptr;  // filter weight of every site, when the plan's filter pass is a general one
   std::vector<Pass> passes;
   FFTTables tables;
 };
 
-}  // namespace
 struct SiteGrid {
   int blocks = 0, spt = 1;  // blocks per configuration, sites per thread
 };
 
+}  // namespace
 
 struct lgf_ctx {
   int n[4];
@@ -211,6 +212,8 @@ lgf_status fail(lgf_ctx *c, lgf_status st, const std::string &msg) {
     lgf_status s_ = (x);         \
     if (s_ != LGF_OK) return s_; \
   } while (0)
+
+unsigned grid1(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
 bool factor_ok(int n) {
   if (n < 2 || n > 1024) return false;
@@ -358,86 +361,116 @@ template <typename T> bool plan_fixed(lgf_ctx *ctx, State<T> &S) {
   return true;
 }
 
-// Plan the FFT passes for element size es (bytes per complex number).
+// Passes for general extents (fft.cuh).
 template <typename T> void plan_passes(lgf_ctx *ctx, State<T> &S) {
   if (!ctx->generic_fft && plan_fixed<T>(ctx, S)) return;
   const int Nx = ctx->n[0], Ny = ctx->n[1], Nz = ctx->n[2], Nt = ctx->n[3];
-  const int64_t Nxy = (int64_t)Nx * Ny, Nxyz = Nxy * Nz;
-  const size_t es = sizeof(cx<T>);
-  const size_t budget = 112 * 1024;  // tile bytes: two blocks per SM
-  const int cmin = (int)std::max<size_t>(1, 64 / es);  // aim for >= 64-byte contiguous runs
-  auto mk = [&](int d0, int d1, int d2, int64_t g0, int64_t g1, int64_t g2, int nb1, int64_t B1, int64_t B2,
-                int nblocks, int nax, int dim0, int mu0, int dim1, int mu1, int mode, int kid) {
-    Pass p{};
-    p.d.d[0] = d0;
-    p.d.d[1] = d1;
-    p.d.d[2] = d2;
-    p.d.g[0] = g0;
-    p.d.g[1] = g1;
-    p.d.g[2] = g2;
-    p.d.nb1 = nb1;
-    p.d.B1 = B1;
-    p.d.B2 = B2;
-    p.d.nblocks = nblocks;
-    p.d.nax = nax;
-    p.d.ax_dim[0] = dim0;
-    p.d.ax_mu[0] = mu0;
-    p.d.ax_dim[1] = dim1;
-    p.d.ax_mu[1] = mu1;
-    p.d.mode = mode;
-    p.kid = kid;
-    const int nel = d0 * d1 * d2;
-    int twn = ctx->n[mu0] + (nax > 1 ? ctx->n[mu1] : 0);
-    p.smem = (size_t)(nel + twn) * es;
-    p.threads = nel >= 2048 ? 512 : 256;
+  const int64_t V = ctx->V;
+  const int es = (int)sizeof(cx<T>);
+  const int64_t want = 2 * (int64_t)ctx->num_sms;  // blocks that a launch should have, when the lattice allows
+  const int64_t per_tile = 4 * (int64_t)ctx->nb;   // blocks per tile: one per packed field and configuration
+  auto phase = [&](Pass &p, int mu, int npen, int A, int B, int S_, int estride) {
+    AxisPhase &a = p.d.ph[p.d.nax++];
+    const AxisFFT &ax = ctx->ax[mu];
+    a.mu = mu;
+    a.N = ax.N;
+    a.nst = ax.nst;
+    int M = ax.N;
+    for (int k = 0; k < ax.nst; ++k) {
+      a.R[k] = ax.R[k];
+      M /= ax.R[k];
+      a.M[k] = fast_div(M);
+    }
+    a.npen = npen;
+    a.A = A;
+    a.B = B;
+    a.S = S_;
+    a.estride = estride;
+    a.dpen = fast_div(npen);
+    a.dA = fast_div(A);
+  };
+  auto finish = [&](Pass &p) {
+    const int nel = p.d.rows * p.d.pitch;
+    int tw = 0;
+    for (int a = 0; a < p.d.nax; ++a) tw += p.d.ph[a].N;
+    p.smem = (size_t)(nel + tw) * es;
+    p.threads = nel >= 4096 ? 512 : 256;
+    p.nblocks = p.d.nblocks;
     return p;
   };
-  auto largest_run = [&](int64_t extent, int64_t per_col_bytes, int cap) {
-    int best = 1;
-    for (int c = 1; c <= cap && c <= extent; ++c)
-      if (extent % c == 0 && (size_t)(c * per_col_bytes) <= budget) best = c;
-    return best;
+  // whole xy planes (or, planes = false, single lattice rows along x), `rows` lattice rows per tile
+  auto row_pass = [&](int rows, bool planes, int mode, int kid) {
+    Pass p{};
+    p.kid = kid;
+    p.d.rowform = 1;
+    p.d.rows = rows;
+    p.d.C = 1;
+    p.d.pitch = Nx | 1;  // odd: the x butterflies of 32 rows fall into different banks
+    p.d.nrow = (unsigned)(V / Nx);
+    p.d.dnx = fast_div(Nx);
+    p.d.mode = mode;
+    p.d.nblocks = (int)((V / Nx + rows - 1) / rows);
+    phase(p, 0, rows, rows, 0, p.d.pitch, 1);
+    if (planes) phase(p, 1, Nx * (rows / Ny), Nx, Ny * p.d.pitch, 1, p.d.pitch);
+    return finish(p);
   };
-  std::vector<Pass> fwd, mid, inv;
-  // x and y
-  if ((size_t)Nxy * es <= budget) {
-    const int nb = Nz * Nt;
-    fwd.push_back(mk(Nx, Ny, 1, 1, Nx, 0, nb, Nxy, 0, nb, 2, 0, 0, 1, 1, 0, KID_FFT_XY_FWD));
-    inv.push_back(mk(Nx, Ny, 1, 1, Nx, 0, nb, Nxy, 0, nb, 2, 0, 0, 1, 1, 1, KID_FFT_XY_INV));
-  } else {
-    const int rows = largest_run(Ny * Nz * Nt, (int64_t)Nx * es, 16);
-    const int nbx = (int)(Ny * (int64_t)Nz * Nt / rows);
-    fwd.push_back(mk(Nx, rows, 1, 1, Nx, 0, nbx, (int64_t)rows * Nx, 0, nbx, 1, 0, 0, 0, 0, 0, KID_FFT_X_FWD));
-    const int cy = largest_run(Nx, (int64_t)Ny * es, 64);
-    const int nby = (Nx / cy) * Nz * Nt;
-    fwd.push_back(mk(cy, Ny, 1, 1, Nx, 0, Nx / cy, cy, Nxy, nby, 1, 1, 1, 0, 0, 0, KID_FFT_Y_FWD));
-    inv.push_back(mk(cy, Ny, 1, 1, Nx, 0, Nx / cy, cy, Nxy, nby, 1, 1, 1, 0, 0, 1, KID_FFT_Y_INV));
-    inv.push_back(mk(Nx, rows, 1, 1, Nx, 0, nbx, (int64_t)rows * Nx, 0, nbx, 1, 0, 0, 0, 0, 1, KID_FFT_X_INV));
-  }
-  // z and t, with the filter
-  const int64_t zt_col = (int64_t)Nz * Nt * es;
-  int czt = 0;
-  for (int c = (int)std::min<int64_t>(Nxy, 64); c >= 1; --c)
-    if (Nxy % c == 0 && (size_t)(c * zt_col) <= budget) {
-      czt = c;
-      break;
+  // C columns of one axis, or (zt) of the z and t axes together
+  auto col_pass = [&](int mu, bool zt, int C, int mode, int kid) {
+    Pass p{};
+    p.kid = kid;
+    p.d.C = C;
+    while ((1 << p.d.logC) < C) ++p.d.logC;
+    p.d.pitch = C;
+    p.d.rows = zt ? Nz * Nt : ctx->n[mu];
+    p.d.rstride = ctx->L.stride[mu];
+    p.d.nin = (unsigned)ctx->L.stride[mu];
+    p.d.ostride = ctx->L.stride[mu] * (zt ? 1 : ctx->n[mu]);
+    p.d.ncol = (unsigned)(V / p.d.rows);
+    p.d.mode = mode;
+    p.d.nblocks = (int)((p.d.ncol + C - 1) / C);
+    if (zt) {
+      phase(p, 2, C * Nt, C, Nz * C, 1, C);
+      phase(p, 3, C * Nz, C, C, 1, Nz * C);
+    } else {
+      phase(p, mu, C, C, 0, 1, C);
     }
-  if (czt >= std::min<int64_t>(cmin, Nxy)) {
-    const int nb = (int)(Nxy / czt);
-    mid.push_back(mk(czt, Nz, Nt, 1, Nxy, Nxyz, nb, czt, 0, nb, 2, 1, 2, 2, 3, 2, KID_FFT_ZT_FILTER));
-  } else {
-    const int cz = largest_run(Nxy, (int64_t)Nz * es, 64);
-    const int nbz = (int)(Nxy / cz) * Nt;
-    fwd.push_back(mk(cz, Nz, 1, 1, Nxy, 0, (int)(Nxy / cz), cz, Nxyz, nbz, 1, 1, 2, 0, 0, 0, KID_FFT_Z_FWD));
-    const int ct = largest_run(Nxyz, (int64_t)Nt * es, 64);
-    const int nbt = (int)(Nxyz / ct);
-    mid.push_back(mk(ct, Nt, 1, 1, Nxyz, 0, nbt, ct, 0, nbt, 1, 1, 3, 0, 0, 2, KID_FFT_T_FILTER));
-    inv.insert(inv.begin(),
-               mk(cz, Nz, 1, 1, Nxy, 0, (int)(Nxy / cz), cz, Nxyz, nbz, 1, 1, 2, 0, 0, 1, KID_FFT_Z_INV));
-  }
+    return finish(p);
+  };
+  // columns per tile: runs of at least 128 bytes, 32 columns where the tile stays within `most` bytes
+  auto cols_for = [&](int64_t rows, int64_t most) {
+    int C = 128 / es;
+    while (C < 32 && 2 * C * rows * es <= most) C *= 2;
+    while (C > 1 && C * rows * es > 160 * 1024) C /= 2;
+    return C;
+  };
   S.passes.clear();
-  for (auto &p : fwd) S.passes.push_back(p);
-  for (auto &p : mid) S.passes.push_back(p);
+  std::vector<Pass> inv;
+  // x and y together while a plane leaves two blocks per SM, several small planes per tile
+  const int64_t plane = (int64_t)Ny * (Nx | 1);
+  if (plane * es <= 96 * 1024) {
+    int G = (int)std::max<int64_t>(1, 2048 / plane);
+    while (G > 1 && (Nz * (int64_t)Nt + G - 1) / G * per_tile < want) --G;
+    S.passes.push_back(row_pass(G * Ny, true, 0, KID_FFT_XY_FWD));
+    inv.push_back(row_pass(G * Ny, true, 1, KID_FFT_XY_INV));
+  } else {
+    const int rows = (int)std::max<int64_t>(1, std::min<int64_t>(32, 48 * 1024 / ((Nx | 1) * es)));
+    const int C = cols_for(Ny, 48 * 1024);
+    S.passes.push_back(row_pass(rows, false, 0, KID_FFT_X_FWD));
+    S.passes.push_back(col_pass(1, false, C, 0, KID_FFT_Y_FWD));
+    inv.push_back(col_pass(1, false, C, 1, KID_FFT_Y_INV));
+    inv.push_back(row_pass(rows, false, 1, KID_FFT_X_INV));
+  }
+  // z and t together while a tile of 128-byte runs leaves two blocks per SM: at 30x20x24x36 (110 KB in float)
+  // 39 us against 23 + 33 + 23 us for z, t with the filter and z again; at 18x12x10x15 (double-float) 19 us
+  // against 9 + 12 + 9 us
+  if ((int64_t)128 * Nz * Nt <= 112 * 1024) {
+    S.passes.push_back(col_pass(2, true, 128 / es, 2, KID_FFT_ZT_FILTER));
+  } else {
+    const int Cz = cols_for(Nz, 48 * 1024), Ct = cols_for(Nt, 48 * 1024);
+    S.passes.push_back(col_pass(2, false, Cz, 0, KID_FFT_Z_FWD));
+    S.passes.push_back(col_pass(3, false, Ct, 2, KID_FFT_T_FILTER));
+    inv.insert(inv.begin(), col_pass(2, false, Cz, 1, KID_FFT_Z_INV));
+  }
   for (auto &p : inv) S.passes.push_back(p);
 }
 
@@ -503,6 +536,29 @@ template <typename T> lgf_status opt_in_smem(lgf_ctx *ctx, State<T> &S) {
   });
 }
 
+// The weight table of a plan whose filter pass reads one (freed when the plan no longer does).
+template <typename T> lgf_status ensure_weights(lgf_ctx *ctx, State<T> &S) {
+  bool need = false;
+  for (auto &p : S.passes) need |= p.kind == 0 && p.d.mode == 2;
+  if (need && !S.weights) {
+    TRY(with_fft_type<T>(ctx, [&](auto tag) -> lgf_status {
+      using FT = decltype(tag);
+      CK(cudaMalloc(&S.weights, sizeof(FT) * (size_t)ctx->V));
+      k_filter_weights<FT><<<grid1(ctx->V, NT), NT, 0, ctx->stream>>>(reinterpret_cast<FT *>(S.weights), ctx->V,
+                                                                     S.tables);
+      CKL();
+      return LGF_OK;
+    }));
+    CK(cudaStreamSynchronize(ctx->stream));  // later passes may run on another stream
+  } else if (!need && S.weights) {
+    CK(cudaStreamSynchronize(ctx->stream));
+    CK(cudaFree(S.weights));
+    S.weights = nullptr;
+  }
+  S.tables.weights = S.weights;
+  return LGF_OK;
+}
+
 template <typename T> lgf_status setup_precision(lgf_ctx *ctx, State<T> &S) {
   const int64_t V = ctx->V;
   const size_t nb = (size_t)ctx->nb;
@@ -531,11 +587,36 @@ template <typename T> lgf_status setup_precision(lgf_ctx *ctx, State<T> &S) {
     }
     S.tables.wscale = ctx->wscale;
     TRY(opt_in_smem<T>(ctx, S));
+    TRY(ensure_weights<T>(ctx, S));
     if constexpr (std::is_same<T, double>::value) {
       CK(cudaFuncSetAttribute(k_update<double, NT_UPDATE64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)update_smem_bytes<NT_UPDATE64>()));
       CK(cudaFuncSetAttribute(k_update<double, NT_UPDATE64>, cudaFuncAttributePreferredSharedMemoryCarveout,
                               (int)cudaSharedmemCarveoutMaxShared));
+    }
+  }
+  return LGF_OK;
+}
+
+// Sites per thread (1 to 4) and blocks of a reducing site kernel, per configuration: the fewest rounds of sites
+// over the waves of blocks, with a block's reduction and start counted as half a round. Four everywhere left
+// most of the GPU idle on small lattices (float Delta at 8^4, 4 blocks: 20.4 us, now 13.3; double at 18x12x10x15:
+// 48 -> 21) and a nearly empty last wave on others (double at 24^3x48: 177 -> 158 us; float at 32^4: 71 -> 67).
+// Without the count for the block, one site per thread would be taken where four are faster (residual Delta at
+// 32^4: 104 against 88 us). One wave of blocks that step through the whole lattice was slower in double (64^4:
+// 5.7 against 3.4 ms).
+lgf_status site_grid(lgf_ctx *ctx, const void *kernel, SiteGrid *g) {
+  int per_sm = 0;
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, 0));
+  const int64_t wave = (int64_t)std::max(per_sm, 1) * ctx->num_sms, chunks = (ctx->V + NT - 1) / NT;
+  double best = 0;
+  for (int spt = 4; spt >= 1; --spt) {
+    const int64_t blocks = (chunks + spt - 1) / spt;
+    const double cost = (double)((blocks * ctx->nb + wave - 1) / wave) * (spt + 0.5);
+    if (best == 0 || cost < best) {
+      best = cost;
+      g->spt = spt;
+      g->blocks = (int)blocks;
     }
   }
   return LGF_OK;
@@ -601,30 +682,6 @@ lgf_status input_ptr(lgf_ctx *ctx, const double *p, size_t bytes, double **buf, 
   TRY(ensure_staging(ctx, buf, have, bytes));
   CK(cudaMemcpyAsync(*buf, p, bytes, cudaMemcpyHostToDevice, ctx->stream));
   *out = *buf;
-// Sites per thread (1 to 4) and blocks of a reducing site kernel, per configuration: the fewest rounds of sites
-// over the waves of blocks, with a block's reduction and start counted as half a round. Four everywhere left
-// most of the GPU idle on small lattices (float Delta at 8^4, 4 blocks: 20.4 us, now 13.3; double at 18x12x10x15:
-// 48 -> 21) and a nearly empty last wave on others (double at 24^3x48: 177 -> 158 us; float at 32^4: 71 -> 67).
-// Without the count for the block, one site per thread would be taken where four are faster (residual Delta at
-// 32^4: 104 against 88 us). One wave of blocks that step through the whole lattice was slower in double (64^4:
-// 5.7 against 3.4 ms).
-lgf_status site_grid(lgf_ctx *ctx, const void *kernel, SiteGrid *g) {
-  int per_sm = 0;
-  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, 0));
-  const int64_t wave = (int64_t)std::max(per_sm, 1) * ctx->num_sms, chunks = (ctx->V + NT - 1) / NT;
-  double best = 0;
-  for (int spt = 4; spt >= 1; --spt) {
-    const int64_t blocks = (chunks + spt - 1) / spt;
-    const double cost = (double)((blocks * ctx->nb + wave - 1) / wave) * (spt + 0.5);
-    if (best == 0 || cost < best) {
-      best = cost;
-      g->spt = spt;
-      g->blocks = (int)blocks;
-    }
-  }
-  return LGF_OK;
-}
-
   return LGF_OK;
 }
 
@@ -643,8 +700,6 @@ lgf_status output_ptr(lgf_ctx *ctx, double *p, size_t bytes, double **buf, size_
   *host = true;
   return LGF_OK;
 }
-
-unsigned grid1(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
 // The kernels that walk along t give each thread kTwalkSlices consecutive t-slices. They run when Nt allows
 // and the launch still has twalk_min_blocks blocks; otherwise the site-order kernels run. Measured: at 64^4
@@ -1225,6 +1280,8 @@ void lgf_destroy(lgf_ctx *ctx) {
   fr(ctx->s32.U);
   fr(ctx->s32.P);
   fr(ctx->s32.G);
+  fr(ctx->s64.weights);
+  fr(ctx->s32.weights);
   for (int mu = 0; mu < 4; ++mu) {
     fr(ctx->s64.tw[mu]);
     fr(ctx->s32.tw[mu]);
