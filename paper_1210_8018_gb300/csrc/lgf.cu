@@ -159,7 +159,7 @@ struct lgf_ctx {
   bool twalk = true;  // float and residual Delta and updates walking along t (LGF_TWALK=0: off; twalk_on)
   int64_t twalk_min_blocks = 2048;  // LGF_TWALK_MIN_BLOCKS
   int handover_split[2] = {2, 2};  // links per site in FP64 (even, odd warps), the rest in fixed point
-  int update_split[2] = {2, 2};    // the same for the general (large-step) form of the double update
+  int update_split[2] = {0, 0};    // the same for the general (large-step) form of the double update
   bool reunit_fp64 = false;    // float stages: periodic projection onto SU(3) in double instead of float
   bool resid_base_ready = false;  // the float link planes hold the double links rounded (by the handover)
   double resid_theta0 = 0;  // theta of the residual stage's base links
@@ -1213,8 +1213,8 @@ static lgf_status create_ctx(const int n[4], int nb, lgf_ctx **out) {
       ctx->handover_split[0] = hs[0] - '0';
       ctx->handover_split[1] = hs[1] - '0';
     }
-    // LGF_UPDATE_SPLIT=ab: the same for the general (large-step) form of the double update (default 22;
-    // 44 is FP64 alone, 00 fixed point alone)
+    // LGF_UPDATE_SPLIT=ab: the same for the general (large-step) form of the double update (default 00,
+    // fixed point alone; 44 is FP64 alone)
     const char *us = std::getenv("LGF_UPDATE_SPLIT");
     if (us && us[0] >= '0' && us[0] <= '4' && us[1] >= '0' && us[1] <= '4') {
       ctx->update_split[0] = us[0] - '0';

@@ -1,5 +1,5 @@
 // q61.cuh -- 64-bit fixed point with 61 fractional bits (Q61) for exact products of SU(3) matrices on the
-// integer pipe (the handover transform of the mixed schedule and the large-step double update).
+// integer pipe (the handover transform of the mixed schedule).
 #pragma once
 #include "su3.cuh"
 

@@ -15,6 +15,7 @@
 #pragma once
 #include <type_traits>
 
+#include "q60.cuh"
 #include "q61.cuh"
 #include "su3.cuh"
 
@@ -688,93 +689,24 @@ __device__ __forceinline__ void update_link_small(double *plane, int64_t V, int6
   st(plane, 8 * V + s, cross_cj(r0[0], r1[1], r0[1], r1[0]));
 }
 
-// General-step update of one link in FP64: rows 0 and 1 of g(x) U g^+(x+mu) by products (g(x) and
-// g(x+mu) from global memory, the link from bu), row 2 = conj(row0 x row1).
+// General-step update of one link (the link from bu, g(x) and g(x+mu) from global memory): in 60-bit fixed
+// point, or in FP64 where `fp64` says so or an entry is out of the fixed-point range.
 template <int NT>
 __device__ __forceinline__ void update_link_general(double *plane, const double *G, int64_t V, int64_t s,
-                                                    int64_t sf, const double2 *bu) {
-  m3<double> t;
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    cx<double> gi[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) gi[k] = ldg(G, (int64_t)(3 * i + k) * V + s);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      cx<double> acc = gi[0] * from_vec<double>(bu[j * NT + threadIdx.x]);
-      acc = cmac(acc, gi[1], from_vec<double>(bu[(3 + j) * NT + threadIdx.x]));
-      acc = cmac(acc, gi[2], from_vec<double>(bu[(6 + j) * NT + threadIdx.x]));
-      t.e[3 * i + j] = acc;
-    }
-  }
-  m3<double> o;
-#pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    const cx<double> h0 = ldg(G, (int64_t)(3 * j) * V + sf);
-    const cx<double> h1 = ldg(G, (int64_t)(3 * j + 1) * V + sf);
-    const cx<double> h2 = ldg(G, (int64_t)(3 * j + 2) * V + sf);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      cx<double> acc = {0, 0};
-      acc = cmac_cj(acc, t.e[3 * i], h0);
-      acc = cmac_cj(acc, t.e[3 * i + 1], h1);
-      acc = cmac_cj(acc, t.e[3 * i + 2], h2);
-      o.e[3 * i + j] = acc;
-    }
-  }
-  store_link(plane, V, s, o);
+                                                    int64_t sf, const double2 *bu, bool fp64) {
+  auto gx = [&](int e) { return ldg(G, (int64_t)e * V + s); };
+  auto u = [&](int e) { return from_vec<double>(bu[e * NT + threadIdx.x]); };
+  auto gy = [&](int e) { return ldg(G, (int64_t)e * V + sf); };
+  auto out = [&](int e, cx<double> v) { st(plane, (int64_t)e * V + s, v); };
+  if (fp64 || !link_product_q60(gx, u, gy, out)) link_product_fp64(gx, u, gy, out);
 }
 
-// The same general-step product in 61-bit fixed point (q61.cuh) on the integer pipe: rows 0 and 1 of
-// g(x) U g^+(x+mu) exact to FP64 rounding, row 2 = conj(row0 x row1) in fixed point.
-template <int NT>
-__device__ __forceinline__ void update_link_general_q(double *plane, const double *G, int64_t V, int64_t s,
-                                                      int64_t sf, const double2 *bu) {
-  cq t[6];
-  {
-    cq gx[6];
-#pragma unroll
-    for (int e = 0; e < 6; ++e) gx[e] = to_cq(ldg(G, (int64_t)e * V + s));
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const cq u0 = to_cq(from_vec<double>(bu[j * NT + threadIdx.x]));
-      const cq u1 = to_cq(from_vec<double>(bu[(3 + j) * NT + threadIdx.x]));
-      const cq u2 = to_cq(from_vec<double>(bu[(6 + j) * NT + threadIdx.x]));
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        cq a = {0, 0};
-        cq_mac(a, gx[3 * i], u0);
-        cq_mac(a, gx[3 * i + 1], u1);
-        cq_mac(a, gx[3 * i + 2], u2);
-        t[3 * i + j] = a;
-      }
-    }
-  }
-  cq o[9];
-#pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    const cq g0 = to_cq(ldg(G, (int64_t)(3 * j) * V + sf));
-    const cq g1 = to_cq(ldg(G, (int64_t)(3 * j + 1) * V + sf));
-    const cq g2 = to_cq(ldg(G, (int64_t)(3 * j + 2) * V + sf));
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      cq a = {0, 0};
-      cq_mac_cj(a, t[3 * i], g0);
-      cq_mac_cj(a, t[3 * i + 1], g1);
-      cq_mac_cj(a, t[3 * i + 2], g2);
-      o[3 * i + j] = a;
-    }
-  }
-  o[6] = cq_cross_cj(o[1], o[5], o[2], o[4]);
-  o[7] = cq_cross_cj(o[2], o[3], o[0], o[5]);
-  o[8] = cq_cross_cj(o[0], o[4], o[1], o[3]);
-#pragma unroll
-  for (int e = 0; e < 9; ++e) st(plane, (int64_t)e * V + s, cx<double>{from_q61(o[e].r), from_q61(o[e].i)});
-}
-
-// Double links: general steps are split between the FP64 pipe (the first fp64_even or fp64_odd directions
-// of a site, in even or odd warps) and the integer pipe (the others, in Q61), so that both pipes work at the
-// same time; both forms are exact to FP64 rounding.
+// Double links: general steps may be split between the FP64 pipe (the first fp64_even or fp64_odd directions
+// of a site, in even or odd warps) and the integer pipe (the others, in Q60); both forms are exact to FP64
+// rounding. All four in Q60 is the fastest: at 24^3 x 48 a general update takes 0.44 ms, against 0.46 with
+// one direction in every other warp in FP64, 0.49 with two in every warp and 0.57 with two in the 61-bit form
+// of q61.cuh, which joins and splits the limbs at every product. The integer and conversion instructions
+// bound it (16 warps per SM, the bytes would take 0.13 ms).
 template <typename T, int NT>
 __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 4 : 2)
     k_update(T *__restrict__ U, const T *__restrict__ G, const float *__restrict__ A, Lattice L, const Ctrl *ctrl,
@@ -836,8 +768,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 4 : 2)
         if (mu < 3) fetch_u<NT>(plane + pstride, V, s, bu0);
       } else {
         const int nf = ((threadIdx.x >> 5) & 1) ? fp64_odd : fp64_even;  // uniform within a warp
-        if (mu < nf) update_link_general<NT>(plane, G, V, s, sf, bu);
-        else update_link_general_q<NT>(plane, G, V, s, sf, bu);
+        update_link_general<NT>(plane, G, V, s, sf, bu, mu < nf);
         if (mu < 3) fetch_link<NT>(plane + pstride, A, V, s, site_fwd(L, s, mu + 1, c[mu + 1]), bu0, bb);
       }
     }
