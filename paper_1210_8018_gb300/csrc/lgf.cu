@@ -123,8 +123,6 @@ struct lgf_ctx {
   double wscale = 0;
   AxisFFT ax[4];
 
-  double *Wev = nullptr;    // differentiable functional: eigenvectors of omega (9 planes)
-  double *lam = nullptr;    // and its eigenvalues (3 planes of doubles)
   double *U0 = nullptr;     // mixed: input links (double planes) for the handover
   float *Gacc = nullptr;    // mixed/float: accumulated gauge transformation (9 float planes)
   float *Rres = nullptr;    // mixed, residual stage: link residual R (4 x 9 float planes)
@@ -135,6 +133,7 @@ struct lgf_ctx {
   size_t staging2_bytes = 0;
   double *partials = nullptr;
   SiteGrid grid64, grid32, grid_resid;  // the reducing site kernels in double, float and the residual stage
+  SiteGrid grid_measure, grid_func;     // k_measure_q60, k_functional_g
   int64_t partials_blocks = 0;  // (theta, F) pairs per configuration in partials
   Ctrl *ctrl = nullptr;
   Ctrl ctrl_host{};
@@ -625,6 +624,8 @@ lgf_status site_grid(lgf_ctx *ctx, const void *kernel, SiteGrid *g) {
 lgf_status ensure_common(lgf_ctx *ctx) {
   if (!ctx->partials) {
     TRY(site_grid(ctx, (const void *)k_delta_f32<NT>, &ctx->grid32));
+    TRY(site_grid(ctx, (const void *)k_measure_q60<NT>, &ctx->grid_measure));
+    TRY(site_grid(ctx, (const void *)k_functional_g<NT>, &ctx->grid_func));
     TRY(with_fft_type<double>(ctx, [&](auto tag) -> lgf_status {
       using FT = decltype(tag);
       TRY(site_grid(ctx, (const void *)k_delta<double, NT, FT>, &ctx->grid64));
@@ -632,7 +633,8 @@ lgf_status ensure_common(lgf_ctx *ctx) {
     }));
     // one (theta, F) pair per block of the largest reducing grid: the site kernels' waves, or the
     // t-walking kernels' columns x Nt / 8 blocks (twalk_on)
-    ctx->partials_blocks = std::max<int64_t>(std::max({ctx->grid64.blocks, ctx->grid32.blocks, ctx->grid_resid.blocks}),
+    ctx->partials_blocks = std::max<int64_t>(std::max({ctx->grid64.blocks, ctx->grid32.blocks, ctx->grid_resid.blocks,
+                                                       ctx->grid_measure.blocks, ctx->grid_func.blocks}),
                                              (ctx->L.stride[3] + NT - 1) / NT * std::max(ctx->n[3] / 8, 1));
     CK(cudaMalloc(&ctx->partials, sizeof(double) * 2 * (size_t)ctx->partials_blocks * ctx->nb));
     CK(cudaMalloc(&ctx->ctrl, sizeof(Ctrl) * ctx->nb));
@@ -1288,8 +1290,6 @@ void lgf_destroy(lgf_ctx *ctx) {
     fr(ctx->p2part[mu]);
   }
   fr(ctx->U0);
-  fr(ctx->Wev);
-  fr(ctx->lam);
   fr(ctx->Gacc);
   fr(ctx->Rres);
   fr(ctx->Kres);
@@ -1523,18 +1523,31 @@ lgf_status lgf_measure(lgf_ctx *ctx, const double *links, double *theta, double 
   const int64_t V = ctx->V;
   const double *src = nullptr;
   TRY(input_ptr(ctx, links, (size_t)4 * V * 9 * 16, &ctx->staging, &ctx->staging_bytes, &src));
-  k_aos_to_planes<double><<<grid1(4 * V, NT), NT, 0, ctx->stream>>>(src, ctx->s64.U, V, 4, 9, 0, 4 * V);
-  CKL();
   memset(&ctx->ctrl_host, 0, sizeof(Ctrl));
   TRY(write_ctrl(ctx));
-  TRY(launch_delta<double>(ctx, ctx->s64, 0, 0));
-  if (plaq) {
-    // stream-ordered after the Delta reduction, which leaves the last-block counter at zero
-    k_plaquette<double, NT><<<ctx->grid64.blocks, NT, 0, ctx->stream>>>(ctx->s64.U, ctx->partials, ctx->ctrl, ctx->L,
-                                                                   ctx->grid64.spt);
-    CKL();
-  }
+  k_links_to_q60<NT><<<grid1(4 * V, NT), NT, 0, ctx->stream>>>(src, reinterpret_cast<int4 *>(ctx->s64.U), V, ctx->ctrl);
+  CKL();
+  // (the packed Delta buffer, which this pass does not need, holds the plaquette partials)
+  k_measure_q60<NT><<<ctx->grid_measure.blocks, NT, 0, ctx->stream>>>(
+      reinterpret_cast<const int4 *>(ctx->s64.U), ctx->partials, ctx->s64.P, ctx->ctrl, ctx->L, ctx->grid_measure.spt,
+      plaq != nullptr);
+  CKL();
   TRY(read_ctrl(ctx));
+  if (ctx->ctrl_host.out_of_range) {
+    // some link is not near SU(3), or not finite: the same in FP64
+    memset(&ctx->ctrl_host, 0, sizeof(Ctrl));
+    TRY(write_ctrl(ctx));
+    k_aos_to_planes<double><<<grid1(4 * V, NT), NT, 0, ctx->stream>>>(src, ctx->s64.U, V, 4, 9, 0, 4 * V);
+    CKL();
+    TRY(launch_delta<double>(ctx, ctx->s64, 0, 0));
+    if (plaq) {
+      // stream-ordered after the Delta reduction, which leaves the last-block counter at zero
+      k_plaquette<double, NT><<<ctx->grid64.blocks, NT, 0, ctx->stream>>>(ctx->s64.U, ctx->partials, ctx->ctrl, ctx->L,
+                                                                         ctx->grid64.spt);
+      CKL();
+    }
+    TRY(read_ctrl(ctx));
+  }
   if (theta) *theta = ctx->ctrl_host.theta;
   if (F) *F = ctx->ctrl_host.F;
   if (plaq) *plaq = ctx->ctrl_host.plaq;
@@ -1760,38 +1773,39 @@ extern "C" lgf_status lgf_update(lgf_ctx *ctx, double *links, const double *g, i
 }
 
 // ------------------------------ differentiable functional ------------------------------
-// Shared set-up of lgf_functional / lgf_functional_grad: links to planes, omega -> g, W, l.
-static lgf_status prepare_functional(lgf_ctx *ctx, const double *links, const double *omega) {
+// Shared set-up of lgf_functional / lgf_functional_grad: the device pointers, and omega -> g in limb planes (in
+// the buffer of the double g).
+constexpr int NT_GRAD = 128;
+static lgf_status prepare_functional(lgf_ctx *ctx, const double *links, const double *omega, const double **ldev,
+                                     const double **odev) {
   TRY(check_ctx(ctx));
   TRY(ensure_common(ctx));
   TRY(setup_precision<double>(ctx, ctx->s64));
   const int64_t V = ctx->V;
-  TRY(alloc(ctx, &ctx->Wev, (size_t)9 * V * 2));
-  TRY(alloc(ctx, &ctx->lam, (size_t)3 * V));
-  const double *ldev = nullptr, *odev = nullptr;
-  TRY(input_ptr(ctx, links, (size_t)4 * V * 144, &ctx->staging, &ctx->staging_bytes, &ldev));
-  TRY(input_ptr(ctx, omega, (size_t)V * 64, &ctx->staging2, &ctx->staging2_bytes, &odev));
-  TRY(to_planes<double>(ctx, ldev, ctx->s64.U, 4));
-  k_expi<NT><<<grid1(V, NT), NT, 0, ctx->stream>>>(odev, ctx->s64.G, ctx->Wev, ctx->lam, V);
+  TRY(input_ptr(ctx, links, (size_t)4 * V * 144, &ctx->staging, &ctx->staging_bytes, ldev));
+  TRY(input_ptr(ctx, omega, (size_t)V * 64, &ctx->staging2, &ctx->staging2_bytes, odev));
+  k_expi<NT><<<grid1(V, NT), NT, 0, ctx->stream>>>(*odev, reinterpret_cast<int4 *>(ctx->s64.G), nullptr, V);
   CKL();
-  ctx->loaded = false;  // the working links were overwritten
+  ctx->loaded = false;  // the working fields were overwritten
   return LGF_OK;
 }
 
 extern "C" lgf_status lgf_functional(lgf_ctx *ctx, const double *links, const double *omega, double *F,
                                      double *g_out) {
-  TRY(prepare_functional(ctx, links, omega));
+  const double *ldev = nullptr, *odev = nullptr;
+  TRY(prepare_functional(ctx, links, omega, &ldev, &odev));
   const int64_t V = ctx->V;
   memset(&ctx->ctrl_host, 0, sizeof(Ctrl));
   TRY(write_ctrl(ctx));
-  k_functional_g<NT><<<ctx->grid64.blocks, NT, 0, ctx->stream>>>(ctx->s64.U, ctx->s64.G, ctx->partials, ctx->ctrl,
-                                                                ctx->L, ctx->grid64.spt);
+  k_functional_g<NT><<<ctx->grid_func.blocks, NT, 0, ctx->stream>>>(
+      ldev, reinterpret_cast<const int4 *>(ctx->s64.G), ctx->partials, ctx->ctrl, ctx->L, ctx->grid_func.spt);
   CKL();
   if (g_out) {
     double *gdev = nullptr;
     bool host = false;
     TRY(output_ptr(ctx, g_out, (size_t)V * 144, &ctx->staging, &ctx->staging_bytes, &gdev, &host));
-    TRY(from_planes<double>(ctx, ctx->s64.G, gdev, 1));
+    k_expi<NT><<<grid1(V, NT), NT, 0, ctx->stream>>>(odev, nullptr, gdev, V);
+    CKL();
     if (host) CK(cudaMemcpyAsync(g_out, gdev, (size_t)V * 144, cudaMemcpyDeviceToHost, ctx->stream));
   }
   TRY(read_ctrl(ctx));
@@ -1801,13 +1815,17 @@ extern "C" lgf_status lgf_functional(lgf_ctx *ctx, const double *links, const do
 
 extern "C" lgf_status lgf_functional_grad(lgf_ctx *ctx, const double *links, const double *omega, double scale,
                                           double *grad) {
-  TRY(prepare_functional(ctx, links, omega));
+  const double *ldev = nullptr, *odev = nullptr;
+  TRY(prepare_functional(ctx, links, omega, &ldev, &odev));
   const int64_t V = ctx->V;
   double *gdev = nullptr;
   bool host = false;
-  TRY(output_ptr(ctx, grad, (size_t)V * 64, &ctx->staging, &ctx->staging_bytes, &gdev, &host));
-  k_functional_grad<NT><<<grid1(V, NT), NT, 0, ctx->stream>>>(ctx->s64.U, ctx->s64.G, ctx->Wev, ctx->lam, gdev,
-                                                              ctx->L, scale);
+  // (a host gradient is gathered in the packed Delta buffer, which has its size and is not needed here)
+  double *packed = ctx->s64.P;
+  size_t packed_bytes = (size_t)V * 64;
+  TRY(output_ptr(ctx, grad, (size_t)V * 64, &packed, &packed_bytes, &gdev, &host));
+  k_functional_grad<NT_GRAD><<<grid1(V, NT_GRAD), NT_GRAD, 0, ctx->stream>>>(
+      ldev, reinterpret_cast<const int4 *>(ctx->s64.G), odev, gdev, ctx->L, scale);
   CKL();
   if (host) CK(cudaMemcpyAsync(grad, gdev, (size_t)V * 64, cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));

@@ -1,5 +1,5 @@
 // q60.cuh -- products of SU(3) matrices in 60-bit fixed point on the integer pipe (the large-step double
-// update).
+// update, the plaquette, the gauge functional and its gradient).
 #pragma once
 #include "su3.cuh"
 
@@ -50,6 +50,48 @@ __device__ __forceinline__ lq lq_split(long long v) { return {(int)(v >> 30), (i
 __device__ __forceinline__ long long lq_join(lq a) { return ((long long)a.h << 30) + a.l; }
 // v 2^-60 rounded to nearest
 __device__ __forceinline__ double q60_double(long long v) { return __ll2double_rn(v) * 0x1p-60; }
+
+// Limb planes: one complex number in 16 bytes.
+__device__ __forceinline__ clq ldg_q(const int4 *p, int64_t idx) {
+  const int4 v = __ldg(p + idx);
+  return {{v.x, v.y}, {v.z, v.w}};
+}
+__device__ __forceinline__ int4 to_int4(clq a) { return make_int4(a.r.h, a.r.l, a.i.h, a.i.l); }
+__device__ __forceinline__ double lq_double(lq a) { return q60_double(lq_join(a)); }
+
+// Rows and columns of at most unit length (to 1.5%): the products of such matrices, and their sums, stay in
+// range whatever the entries are. Gathered one element at a time (|x| < 2 each: 14-bit squares, 31-bit sums).
+struct unit_check {
+  int row[3] = {0, 0, 0}, col[3] = {0, 0, 0};
+  __device__ __forceinline__ void add(int i, int j, clq a) {
+    const int x = a.r.h >> 17, y = a.i.h >> 17, n = x * x + y * y;
+    row[i] += n;
+    col[j] += n;
+  }
+  __device__ __forceinline__ bool ok(unsigned top) const {
+    constexpr int limit = 69000000;  // 2^26 is a unit vector
+    return lq_in_range(top) &&
+           max(max(max(row[0], row[1]), row[2]), max(max(col[0], col[1]), col[2])) <= limit;
+  }
+};
+
+// acc += a b, += a conj(b)
+struct clacc {
+  lacc re, im;
+};
+__device__ __forceinline__ void clmac(clacc &s, clq a, clq b) {
+  lmac(s.re, a.r, b.r);
+  lmac(s.re, a.i, lq_neg(b.i));
+  lmac(s.im, a.r, b.i);
+  lmac(s.im, a.i, b.r);
+}
+__device__ __forceinline__ void clmac_cj(clacc &s, clq a, clq b) {
+  lmac(s.re, a.r, b.r);
+  lmac(s.re, a.i, b.i);
+  lmac(s.im, a.i, b.r);
+  lmac(s.im, a.r, lq_neg(b.i));
+}
+__device__ __forceinline__ clq clacc_split(const clacc &s) { return {lq_split(lacc_value(s.re)), lq_split(lacc_value(s.im))}; }
 
 // The link g(x) U g^+(x + mu): rows 0 and 1 by products, row 2 = conj(row0 x row1). gx_of, u_of and g_of give
 // the elements of g(x) (rows 0-1 are used), U and g(x + mu); out(e, value) is called for the nine elements,

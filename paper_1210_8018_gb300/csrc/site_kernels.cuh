@@ -45,6 +45,7 @@ struct Ctrl {
                          // mixed schedule; kernels of another stage return at once (a batch launches
                          // the float and the double kernels in the mixed schedule)
   double plaq;           // average plaquette, written by k_plaquette
+  int out_of_range;      // 1 when a link of k_links_to_q60 cannot be held in 60-bit fixed point
 };
 constexpr int kStageResidual = 2;
 
@@ -137,8 +138,9 @@ template <int NT> __device__ __forceinline__ void block_sum2(double &a, double &
 // fixed order and updates the loop control (Algorithm 1: "calculate Delta(x), F and theta", then the
 // while-test theta >= eps). f_offset is added to F (the residual stage sums only the residual's traces).
 // The block's number among the grid's nblk blocks is bid (blockIdx.x for one-dimensional grids).
+// Returns true in the last block.
 template <int NT>
-__device__ __forceinline__ void reduce_and_finalize_at(double th, double f, double *partials, Ctrl *ctrl, int64_t V,
+__device__ __forceinline__ bool reduce_and_finalize_at(double th, double f, double *partials, Ctrl *ctrl, int64_t V,
                                                        int counts_update, double f_offset, unsigned bid,
                                                        unsigned nblk) {
   __shared__ bool last;
@@ -150,7 +152,7 @@ __device__ __forceinline__ void reduce_and_finalize_at(double th, double f, doub
     last = (atomicAdd(&ctrl->ticket, 1u) == nblk - 1);
   }
   __syncthreads();
-  if (!last) return;
+  if (!last) return false;
   __threadfence();
   double a = 0.0, b = 0.0;
   for (unsigned k = threadIdx.x; k < nblk; k += NT) {
@@ -178,6 +180,7 @@ __device__ __forceinline__ void reduce_and_finalize_at(double th, double f, doub
       ctrl->active = (theta >= ctrl->threshold) && (it < ctrl->limit);
     }
   }
+  return true;
 }
 template <int NT>
 __device__ __forceinline__ void reduce_and_finalize(double th, double f, double *partials, Ctrl *ctrl, int64_t V,
@@ -933,6 +936,128 @@ __global__ void __launch_bounds__(NT) k_plaquette(const T *__restrict__ U, doubl
     ctrl->plaq = a / (3.0 * 6.0 * (double)V);  // (1/3) Re Tr over V sites and 6 planes
     ctrl->ticket = 0;
   }
+}
+
+// The caller's links in limb planes Q[(mu*9 + e)*V + s] (q60.cuh) for k_measure_q60.
+template <int NT>
+__global__ void __launch_bounds__(NT) k_links_to_q60(const double *__restrict__ A, int4 *__restrict__ Q, int64_t V,
+                                                    Ctrl *ctrl) {
+  const int64_t idx = (int64_t)blockIdx.x * NT + threadIdx.x;
+  if (idx >= 4 * V) return;
+  const int64_t mu = idx / V, s = idx - mu * V;
+  const double2 *src = reinterpret_cast<const double2 *>(A) + idx * 9;
+  unsigned top = 0;
+  unit_check unit;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    const clq v = to_clq(from_vec<double>(src[e]), top);
+    unit.add(e / 3, e % 3, v);
+    Q[(mu * 9 + e) * V + s] = to_int4(v);
+  }
+  if (!unit.ok(top)) ctrl->out_of_range = 1;
+}
+
+// theta, F and (with_plaq) the average plaquette of the links in limb planes, in one pass: the sums of Delta
+// in 56-bit fixed point as in k_delta, the products of the plaquettes in Q60. In FP64 the plaquettes are
+// 1400 multiply-adds per site on a pipe that does two per SM and clock (48^3 x 40: 10.6 ms); here they are
+// 4200 integer multiply-adds, 32 per SM and clock. The matrices are read a row at a time, again from L1
+// where a row is needed three times, which keeps more warps in flight than holding them in registers.
+template <int NT>
+__global__ void __launch_bounds__(NT, 2) k_measure_q60(const int4 *__restrict__ Q, double *partials, double *plaq_part,
+                                                      Ctrl *ctrl, Lattice L, int spt, int with_plaq) {
+  const int64_t V = L.V;
+  double th = 0.0, f = 0.0, pl = 0.0;
+#pragma unroll 1
+  for (int n = 0; n < spt; ++n) {
+    const int64_t s = ((int64_t)blockIdx.x * spt + n) * NT + threadIdx.x;
+    if (s >= V) break;
+    int c[4];
+    site_coords(L, s, c);
+    {
+      long long acc[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, tr = 0;
+      auto q56 = [](lq a) { return ((long long)a.h << 26) + (a.l >> 4); };
+#pragma unroll 1
+      for (int mu = 0; mu < 4; ++mu) {
+        const int4 *plane = Q + (int64_t)mu * 9 * V;
+#pragma unroll
+        for (int back = 1; back >= 0; --back) {  // + U_mu(x - mu), - U_mu(x)
+          const int64_t at = back ? site_back(L, s, mu, c[mu]) : s;
+          clq u[9];
+#pragma unroll
+          for (int e = 0; e < 9; ++e) u[e] = ldg_q(plane, (int64_t)e * V + at);
+          const long long t[9] = {q56(u[1].r) - q56(u[3].r), q56(u[1].i) + q56(u[3].i), q56(u[2].r) - q56(u[6].r),
+                                  q56(u[2].i) + q56(u[6].i), q56(u[5].r) - q56(u[7].r), q56(u[5].i) + q56(u[7].i),
+                                  q56(u[0].i),               q56(u[4].i),               q56(u[8].i)};
+#pragma unroll
+          for (int k = 0; k < 9; ++k) acc[k] += back ? t[k] : -t[k];
+          if (!back) tr += ((lq_join(u[0].r) >> 2) + (lq_join(u[4].r) >> 2)) + (lq_join(u[8].r) >> 2);
+        }
+      }
+      constexpr double sc = 0x1p-56, w = 2.0 / 3.0 * sc;
+      const long long sd = acc[6] + acc[7] + acc[8];
+      double off = 0, dia = 0;
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        const double d = __ll2double_rn(acc[k]) * sc;
+        off = fma(d, d, off);
+      }
+#pragma unroll
+      for (int k = 6; k < 9; ++k) {
+        const double d = __ll2double_rn(3 * acc[k] - sd) * w;
+        dia = fma(d, d, dia);
+      }
+      th += fma(2.0, off, dia);
+      f += __ll2double_rn(tr) * 0x1p-58;
+    }
+    if (!with_plaq) continue;
+#pragma unroll 1
+    for (int mu = 0; mu < 3; ++mu)
+#pragma unroll 1
+      for (int nu = mu + 1; nu < 4; ++nu) {
+        // Re Tr [U_mu(x) U_nu(x+mu)] [U_nu(x) U_mu(x+nu)]^+, one row of the two products at a time
+        const int4 *pa = Q + (int64_t)mu * 9 * V, *pb = Q + (int64_t)nu * 9 * V;
+        const int64_t smu = site_fwd(L, s, mu, c[mu]), snu = site_fwd(L, s, nu, c[nu]);
+        long long sum = 0;
+#pragma unroll 1
+        for (int i = 0; i < 3; ++i) {
+          auto row_of = [&](const int4 *a, const int4 *b, int64_t sb, clq row[3]) {
+            clacc t[3] = {};
+#pragma unroll 1
+            for (int k = 0; k < 3; ++k) {
+              const clq x = ldg_q(a, (int64_t)(3 * i + k) * V + s);
+#pragma unroll
+              for (int j = 0; j < 3; ++j) clmac(t[j], x, ldg_q(b, (int64_t)(3 * k + j) * V + sb));
+            }
+#pragma unroll
+            for (int j = 0; j < 3; ++j) row[j] = clacc_split(t[j]);
+          };
+          clq t[3], w[3];
+          row_of(pa, pb, smu, t);
+          row_of(pb, pa, snu, w);
+          lacc dot = {};
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            lmac(dot, t[j].r, w[j].r);
+            lmac(dot, t[j].i, w[j].i);
+          }
+          sum += lacc_value(dot);
+        }
+        pl += q60_double(sum);
+      }
+  }
+  if (with_plaq) {
+    double zero = 0.0;
+    block_sum2<NT>(pl, zero);
+    if (threadIdx.x == 0) plaq_part[blockIdx.x] = pl;
+    __syncthreads();
+  }
+  // (thread 0 wrote the plaquette partial before the fence and the ticket of the reduction)
+  if (!reduce_and_finalize_at<NT>(th, f, partials, ctrl, V, 0, 0.0, blockIdx.x, gridDim.x) || !with_plaq) return;
+  double a = 0.0, b = 0.0;
+  for (unsigned k = threadIdx.x; k < gridDim.x; k += NT) a += __ldcg(plaq_part + k);
+  __syncthreads();
+  block_sum2<NT>(a, b);
+  if (threadIdx.x == 0) ctrl->plaq = a / (3.0 * 6.0 * (double)V);
 }
 
 }  // namespace lgf
