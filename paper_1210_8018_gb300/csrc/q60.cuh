@@ -93,77 +93,26 @@ __device__ __forceinline__ void clmac_cj(clacc &s, clq a, clq b) {
 }
 __device__ __forceinline__ clq clacc_split(const clacc &s) { return {lq_split(lacc_value(s.re)), lq_split(lacc_value(s.im))}; }
 
-// The link g(x) U g^+(x + mu): rows 0 and 1 by products, row 2 = conj(row0 x row1). gx_of, u_of and g_of give
-// the elements of g(x) (rows 0-1 are used), U and g(x + mu); out(e, value) is called for the nine elements,
-// unless some lane of the warp has an entry out of range: then nothing is written and the answer is false.
-// The lanes that are active in a warp call it together.
-template <typename XOf, typename UOf, typename GOf, typename Out>
-__device__ __forceinline__ bool link_product_q60(XOf gx_of, UOf u_of, GOf g_of, Out out) {
-  unsigned top = 0;
-  clq gx[6];
-#pragma unroll
-  for (int e = 0; e < 6; ++e) gx[e] = to_clq(gx_of(e), top);
-  clq t[6];  // rows 0-1 of g(x) U, one column of U at a time
-#pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    lacc re[2] = {}, im[2] = {};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const clq u = to_clq(u_of(3 * k + j), top);
-      const lq ni = lq_neg(u.i);
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        lmac(re[i], gx[3 * i + k].r, u.r);
-        lmac(re[i], gx[3 * i + k].i, ni);
-        lmac(im[i], gx[3 * i + k].r, u.i);
-        lmac(im[i], gx[3 * i + k].i, u.r);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) t[3 * i + j] = {lq_split(lacc_value(re[i])), lq_split(lacc_value(im[i]))};
-  }
-  clq o[6];  // rows 0-1 of the result
-#pragma unroll
-  for (int j = 0; j < 3; ++j) {  // one row of g(x + mu) at a time
-    lacc re[2] = {}, im[2] = {};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const clq g = to_clq(g_of(3 * j + k), top);
-      const lq ni = lq_neg(g.i);
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        lmac(re[i], t[3 * i + k].r, g.r);
-        lmac(re[i], t[3 * i + k].i, g.i);
-        lmac(im[i], t[3 * i + k].i, g.r);
-        lmac(im[i], t[3 * i + k].r, ni);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-      o[3 * i + j] = {lq_split(lacc_value(re[i])), lq_split(lacc_value(im[i]))};
-  }
-  if (__any_sync(__activemask(), !lq_in_range(top))) return false;
-#pragma unroll
-  for (int e = 0; e < 6; ++e) out(e, cx<double>{q60_double(lq_join(o[e].r)), q60_double(lq_join(o[e].i))});
-#pragma unroll
-  for (int e = 6; e < 9; ++e) {  // conj(a b - c d)
-    const clq a = o[e == 6 ? 1 : e == 7 ? 2 : 0], b = o[e == 6 ? 5 : e == 7 ? 3 : 4];
-    const clq c = o[e == 6 ? 2 : e == 7 ? 0 : 1], d = o[e == 6 ? 4 : e == 7 ? 5 : 3];
-    lacc re = {}, im = {};
-    lmac(re, a.r, b.r);
-    lmac(re, a.i, lq_neg(b.i));
-    lmac(re, c.r, lq_neg(d.r));
-    lmac(re, c.i, d.i);
-    lmac(im, a.r, lq_neg(b.i));
-    lmac(im, a.i, lq_neg(b.r));
-    lmac(im, c.r, d.i);
-    lmac(im, c.i, d.r);
-    out(e, cx<double>{q60_double(lacc_value(re)), q60_double(lacc_value(im))});
-  }
-  return true;
+// The words of a complex double (x: re lo, y: re hi, z: im lo, w: im hi) as limbs, by floor(x 2^60) - 0 or 1 (a
+// negative number is the complement of its truncated magnitude): nine operations a number fewer than a
+// conversion that truncates, for callers who have checked the range.
+__device__ __forceinline__ lq words_lq(unsigned hi, unsigned lo) {
+  const unsigned long long m =
+      ((unsigned long long)((__funnelshift_l(lo, hi, 8) & 0x0FFFFFFFu) | 0x10000000u) << 32) | (lo << 8);
+  const unsigned long long q = m >> min((0x3FFFFFFFu - (hi & 0x7FFFFFFFu)) >> 20, 63u);
+  const unsigned sg = (unsigned)((int)hi >> 31);
+  return {(int)((unsigned)(q >> 30) ^ sg), (int)(((unsigned)q ^ sg) & 0x3FFFFFFFu)};
 }
+__device__ __forceinline__ clq words_clq(int4 v) {
+  return {words_lq((unsigned)v.y, (unsigned)v.x), words_lq((unsigned)v.w, (unsigned)v.z)};
+}
+__device__ __forceinline__ cx<double> words_double(int4 v) {
+  return {__hiloint2double(v.y, v.x), __hiloint2double(v.w, v.z)};
+}
+__device__ __forceinline__ clq limbs_of(int4 v) { return {{v.x, v.y}, {v.z, v.w}}; }
 
-// The same in FP64, for entries of any size.
+// The link g(x) U g^+(x + mu) in FP64: rows 0 and 1 by products, row 2 = conj(row0 x row1). gx_of, u_of and
+// g_of give the elements of g(x) (rows 0-1 are used), U and g(x + mu); out(e, value) takes the nine elements.
 template <typename XOf, typename UOf, typename GOf, typename Out>
 __device__ __forceinline__ void link_product_fp64(XOf gx_of, UOf u_of, GOf g_of, Out out) {
   m3<double> t, o;

@@ -570,7 +570,8 @@ template <int NT> __global__ void k_a_from_g(const double *__restrict__ G, float
 // ---------------------------------------------------------------------------------------------
 // a7: U_mu(x) -> g(x) U_mu(x) g^dagger(x + mu) for the four directions.
 //
-// Double links take one of two forms of the same product, chosen per warp and per link:
+// Double links take one of two forms of the same product, chosen per warp: the small-step form for the
+// directions before the first that does not allow it, the general form from there on:
 //  * small step: with g(x) = 1 + a and g(x+mu) = 1 + b, rows 0 and 1 of the new link are U + delta with
 //      delta = a U + (U + a U) b^dagger,
 //    delta formed in double-float arithmetic (FP32 operations, ~2^-48 relative) and added to U in
@@ -578,7 +579,7 @@ template <int NT> __global__ void k_a_from_g(const double *__restrict__ G, float
 //    2^-48 |a| |U|) is at or below the FP64 rounding of the product itself, and the FP64 pipe -- 1/64
 //    of the FP32 rate on this GPU -- does only the final additions. Near convergence |a| ~ alpha |Delta|
 //    is far below the bound.
-//  * general step: rows 0 and 1 of g(x) U g^+(x+mu) by FP64 products, row 2 = conj(row0 x row1).
+//  * general step: rows 0 and 1 of g(x) U g^+(x+mu) by products exact to FP64 rounding, row 2 = conj(row0 x row1).
 // ---------------------------------------------------------------------------------------------
 constexpr int kSmallStepFloatExpField = 127 - 8;  // |x| < 2^-7  <=>  float exponent field of hi <= 119
 
@@ -692,16 +693,102 @@ __device__ __forceinline__ void update_link_small(double *plane, int64_t V, int6
   st(plane, 8 * V + s, cross_cj(r0[0], r1[1], r0[1], r1[0]));
 }
 
-// General-step update of one link (the link from bu, g(x) and g(x+mu) from global memory): in 60-bit fixed
-// point, or in FP64 where `fp64` says so or an entry is out of the fixed-point range.
+// General-step update of the links mu0 .. 3 of a site: rows 0 and 1 of g(x) U g^+(x+mu) in 60-bit fixed
+// point (q60.cuh), row 2 = conj(row0 x row1); in FP64 for the directions below nf and where an entry of the
+// warp is out of the fixed-point range. `cur` holds the first link and is with `oth` and `gs` nine slots each
+// per thread: the loops over columns are rolled and keep the limbs of g(x) U (in oth) and of the result (in
+// cur) in shared memory, because the unrolled form, 3000 instructions a link, waited for its own code. While
+// row 2 is formed the next link and g are copied to oth and gs.
 template <int NT>
-__device__ __forceinline__ void update_link_general(double *plane, const double *G, int64_t V, int64_t s,
-                                                    int64_t sf, const double2 *bu, bool fp64) {
-  auto gx = [&](int e) { return ldg(G, (int64_t)e * V + s); };
-  auto u = [&](int e) { return from_vec<double>(bu[e * NT + threadIdx.x]); };
-  auto gy = [&](int e) { return ldg(G, (int64_t)e * V + sf); };
-  auto out = [&](int e, cx<double> v) { st(plane, (int64_t)e * V + s, v); };
-  if (fp64 || !link_product_q60(gx, u, gy, out)) link_product_fp64(gx, u, gy, out);
+__device__ __forceinline__ void update_links_general(double *U, const double *G, const Lattice &L, int64_t s,
+                                                     const int c[4], int mu0, int nf, int4 *cur, int4 *oth,
+                                                     int4 *gs) {
+  const int64_t V = L.V, pstride = link_plane_stride<double>(V);
+  cur += threadIdx.x;
+  oth += threadIdx.x;
+  gs += threadIdx.x;
+  auto fetch = [&](const double *src, int64_t at, int4 *dst) {
+    const int4 *p = reinterpret_cast<const int4 *>(src) + at;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) cp_async16(dst + e * NT, p + (int64_t)e * V);
+    cp_async_commit();
+  };
+  const int4 *gp = reinterpret_cast<const int4 *>(G) + s;
+  fetch(G, site_fwd(L, s, mu0, c[mu0]), gs);
+  clq gx[6];
+  int topx = 0;
+#pragma unroll
+  for (int e = 0; e < 6; ++e) {
+    const int4 v = __ldg(gp + (int64_t)e * V);
+    topx |= v.y | v.w;
+    gx[e] = words_clq(v);
+  }
+#pragma unroll 1
+  for (int mu = mu0; mu < 4; ++mu) {
+    double *plane = U + (int64_t)mu * pstride;
+    auto out = [&](int e, cx<double> v) { st(plane, (int64_t)e * V + s, v); };
+    auto next = [&]() {
+      if (mu == 3) return;
+      fetch(plane + pstride, s, oth);
+      fetch(G, site_fwd(L, s, mu + 1, c[mu + 1]), gs);
+    };
+    cp_async_wait_all();
+    int top = topx;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      top |= cur[e * NT].y | cur[e * NT].w;
+      top |= gs[e * NT].y | gs[e * NT].w;
+    }
+    if (__any_sync(__activemask(), mu < nf || (top & 0x40000000))) {  // bit 30: a magnitude of 2 or more
+      link_product_fp64([&](int e) { return words_double(__ldg(gp + (int64_t)e * V)); },
+                        [&](int e) { return words_double(cur[e * NT]); },
+                        [&](int e) { return words_double(gs[e * NT]); }, out);
+      next();
+    } else {
+#pragma unroll 1
+      for (int j = 0; j < 3; ++j) {  // column j of rows 0-1 of g(x) U
+        clacc t[2] = {};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const clq u = words_clq(cur[(3 * k + j) * NT]);
+#pragma unroll
+          for (int i = 0; i < 2; ++i) clmac(t[i], gx[3 * i + k], u);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) oth[(3 * i + j) * NT] = to_int4(clacc_split(t[i]));
+      }
+#pragma unroll 1
+      for (int j = 0; j < 3; ++j) {  // column j of rows 0-1 of the result, from row j of g(x + mu)
+        clacc t[2] = {};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const clq g = words_clq(gs[(3 * j + k) * NT]);
+#pragma unroll
+          for (int i = 0; i < 2; ++i) clmac_cj(t[i], limbs_of(oth[(3 * i + k) * NT]), g);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const long long vr = lacc_value(t[i].re), vi = lacc_value(t[i].im);
+          cur[(3 * i + j) * NT] = to_int4({lq_split(vr), lq_split(vi)});
+          out(3 * i + j, {q60_double(vr), q60_double(vi)});
+        }
+      }
+      next();
+#pragma unroll 1
+      for (int j = 0; j < 3; ++j) {
+        const int j1 = j == 2 ? 0 : j + 1, j2 = j == 0 ? 2 : j - 1;
+        const clq a = limbs_of(cur[j1 * NT]), b = limbs_of(cur[(3 + j2) * NT]);
+        const clq d = limbs_of(cur[j2 * NT]), e = limbs_of(cur[(3 + j1) * NT]);
+        clacc t = {};  // a b - d e
+        clmac(t, a, b);
+        clmac(t, d, {lq_neg(e.r), lq_neg(e.i)});
+        out(6 + j, {q60_double(lacc_value(t.re)), q60_double(-lacc_value(t.im))});
+      }
+    }
+    int4 *const swap = cur;
+    cur = oth;
+    oth = swap;
+  }
 }
 
 // Double links: general steps may be split between the FP64 pipe (the first fp64_even or fp64_odd directions
@@ -746,35 +833,35 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 4 : 2)
     int ea = 0;
 #pragma unroll
     for (int e = 0; e < 9; ++e) ea = exp_max_df(from_vec<df64>(sa[e * NT + threadIdx.x]), ea);
+    // small-step links up to the first that has a large a or b; the general form takes the rest
+    int mu = 0;
 #pragma unroll 1
-    for (int mu = 0; mu < 4; ++mu) {
+    for (; mu < 4; ++mu) {
+      if (__any_sync(__activemask(), !allow_small || ea > kSmallStepFloatExpField)) break;
       double *plane = U + (int64_t)mu * pstride;
-      const double2 *bu = bu0;
       cp_async_wait_all();
       cx<df64> b[9];
-      int eb = ea;
+      int eb = 0;
 #pragma unroll
       for (int e = 0; e < 9; ++e) {
         b[e] = from_vec<df64>(bb[e * NT + threadIdx.x]);
         eb = exp_max_df(b[e], eb);
       }
-      const int64_t sf = site_fwd(L, s, mu, c[mu]);
-      if (__all_sync(__activemask(), allow_small && eb <= kSmallStepFloatExpField)) {
-        cx<df64> u[9];
+      if (__any_sync(__activemask(), eb > kSmallStepFloatExpField)) break;
+      cx<df64> u[9];
 #pragma unroll
-        for (int e = 0; e < 9; ++e) {
-          const double2 v = bu[e * NT + threadIdx.x];
-          u[e] = {df64_split_fast(v.x), df64_split_fast(v.y)};
-        }
-        if (mu < 3) fetch_b<NT>(A, V, site_fwd(L, s, mu + 1, c[mu + 1]), bb);
-        update_link_small<NT>(plane, V, s, sa, bu0, u, b);
-        if (mu < 3) fetch_u<NT>(plane + pstride, V, s, bu0);
-      } else {
-        const int nf = ((threadIdx.x >> 5) & 1) ? fp64_odd : fp64_even;  // uniform within a warp
-        update_link_general<NT>(plane, G, V, s, sf, bu, mu < nf);
-        if (mu < 3) fetch_link<NT>(plane + pstride, A, V, s, site_fwd(L, s, mu + 1, c[mu + 1]), bu0, bb);
+      for (int e = 0; e < 9; ++e) {
+        const double2 v = bu0[e * NT + threadIdx.x];
+        u[e] = {df64_split_fast(v.x), df64_split_fast(v.y)};
       }
+      if (mu < 3) fetch_b<NT>(A, V, site_fwd(L, s, mu + 1, c[mu + 1]), bb);
+      update_link_small<NT>(plane, V, s, sa, bu0, u, b);
+      if (mu < 3) fetch_u<NT>(plane + pstride, V, s, bu0);
     }
+    if (mu < 4)
+      update_links_general<NT>(U, G, L, s, c, mu, ((threadIdx.x >> 5) & 1) ? fp64_odd : fp64_even,
+                               reinterpret_cast<int4 *>(bu0), reinterpret_cast<int4 *>(sa),
+                               reinterpret_cast<int4 *>(bb));
   } else {
     m3<T> gx;
 #pragma unroll
