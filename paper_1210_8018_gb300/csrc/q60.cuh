@@ -93,15 +93,15 @@ __device__ __forceinline__ void clmac_cj(clacc &s, clq a, clq b) {
 }
 __device__ __forceinline__ clq clacc_split(const clacc &s) { return {lq_split(lacc_value(s.re)), lq_split(lacc_value(s.im))}; }
 
-// The words of a complex double (x: re lo, y: re hi, z: im lo, w: im hi) as limbs, by floor(x 2^60) - 0 or 1 (a
-// negative number is the complement of its truncated magnitude): nine operations a number fewer than a
-// conversion that truncates, for callers who have checked the range.
+// The words of a complex double (x: re lo, y: re hi, z: im lo, w: im hi) as limbs, for callers who have checked
+// the range. The sign is exact: a complement alone would save two operations of sixteen, but lengthens every
+// negative number by 2^-60, and the links with it, a little in each update.
 __device__ __forceinline__ lq words_lq(unsigned hi, unsigned lo) {
   const unsigned long long m =
       ((unsigned long long)((__funnelshift_l(lo, hi, 8) & 0x0FFFFFFFu) | 0x10000000u) << 32) | (lo << 8);
-  const unsigned long long q = m >> min((0x3FFFFFFFu - (hi & 0x7FFFFFFFu)) >> 20, 63u);
-  const unsigned sg = (unsigned)((int)hi >> 31);
-  return {(int)((unsigned)(q >> 30) ^ sg), (int)(((unsigned)q ^ sg) & 0x3FFFFFFFu)};
+  const long long q = (long long)(m >> min((0x3FFFFFFFu - (hi & 0x7FFFFFFFu)) >> 20, 63u));
+  const long long v = (int)hi < 0 ? -q : q;
+  return {(int)(v >> 30), (int)((unsigned)v & 0x3FFFFFFFu)};
 }
 __device__ __forceinline__ clq words_clq(int4 v) {
   return {words_lq((unsigned)v.y, (unsigned)v.x), words_lq((unsigned)v.w, (unsigned)v.z)};
