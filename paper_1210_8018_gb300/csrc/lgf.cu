@@ -133,7 +133,7 @@ struct lgf_ctx {
   size_t staging2_bytes = 0;
   double *partials = nullptr;
   SiteGrid grid64, grid32, grid_resid;  // the reducing site kernels in double, float and the residual stage
-  SiteGrid grid_measure, grid_func;     // k_measure_q60, k_functional_g
+  SiteGrid grid_measure, grid_func, grid_matrices;  // k_measure_q60, k_functional_g, k_delta_matrices
   int64_t partials_blocks = 0;  // (theta, F) pairs per configuration in partials
   Ctrl *ctrl = nullptr;
   Ctrl ctrl_host{};
@@ -626,6 +626,7 @@ lgf_status ensure_common(lgf_ctx *ctx) {
     TRY(site_grid(ctx, (const void *)k_delta_f32<NT>, &ctx->grid32));
     TRY(site_grid(ctx, (const void *)k_measure_q60<NT>, &ctx->grid_measure));
     TRY(site_grid(ctx, (const void *)k_functional_g<NT>, &ctx->grid_func));
+    TRY(site_grid(ctx, (const void *)k_delta_matrices<NT>, &ctx->grid_matrices));
     TRY(with_fft_type<double>(ctx, [&](auto tag) -> lgf_status {
       using FT = decltype(tag);
       TRY(site_grid(ctx, (const void *)k_delta<double, NT, FT>, &ctx->grid64));
@@ -634,7 +635,8 @@ lgf_status ensure_common(lgf_ctx *ctx) {
     // one (theta, F) pair per block of the largest reducing grid: the site kernels' waves, or the
     // t-walking kernels' columns x Nt / 8 blocks (twalk_on)
     ctx->partials_blocks = std::max<int64_t>(std::max({ctx->grid64.blocks, ctx->grid32.blocks, ctx->grid_resid.blocks,
-                                                       ctx->grid_measure.blocks, ctx->grid_func.blocks}),
+                                                       ctx->grid_measure.blocks, ctx->grid_func.blocks,
+                                                       ctx->grid_matrices.blocks}),
                                              (ctx->L.stride[3] + NT - 1) / NT * std::max(ctx->n[3] / 8, 1));
     CK(cudaMalloc(&ctx->partials, sizeof(double) * 2 * (size_t)ctx->partials_blocks * ctx->nb));
     CK(cudaMalloc(&ctx->ctrl, sizeof(Ctrl) * ctx->nb));
@@ -1578,18 +1580,25 @@ template <typename T> static lgf_status unpack_field(lgf_ctx *ctx, State<T> &S, 
 template <typename T> static lgf_status step_delta(lgf_ctx *ctx, State<T> &S, const double *src, double *dst,
                                                    double *theta, double *F) {
   const int64_t V = ctx->V;
-  k_aos_to_planes<T><<<grid1(4 * V, NT), NT, 0, ctx->stream>>>(src, S.U, V, 4, LinkStore<T>::planes, 0, 4 * V);
-  CKL();
   memset(&ctx->ctrl_host, 0, sizeof(Ctrl));
   TRY(write_ctrl(ctx));
   if constexpr (std::is_same<T, double>::value) {
-    // the caller gets Delta in full FP64: pack it as double, not as the type of the double path's FFT
-    k_delta<double, NT, double><<<dim3(ctx->grid64.blocks, 1, 1), NT, 0, ctx->stream>>>(
-        S.U, S.P, ctx->partials, ctx->ctrl, ctx->L, 0, 0, kid<T>(KID_DELTA), ctx->grid64.spt);
-    CKL();
-    k_unpack_antiherm<double><<<grid1(V, NT), NT, 0, ctx->stream>>>(S.P, dst, V);
-    CKL();
+    if (dst + (size_t)18 * V <= src || src + (size_t)72 * V <= dst) {
+      k_delta_matrices<NT><<<ctx->grid_matrices.blocks, NT, 0, ctx->stream>>>(src, dst, ctx->partials, ctx->ctrl, ctx->L,
+                                                                             ctx->grid_matrices.spt);
+      CKL();
+    } else {  // Delta goes over some of the links: through the planes, packed in full FP64
+      k_aos_to_planes<T><<<grid1(4 * V, NT), NT, 0, ctx->stream>>>(src, S.U, V, 4, LinkStore<T>::planes, 0, 4 * V);
+      CKL();
+      k_delta<double, NT, double><<<dim3(ctx->grid64.blocks, 1, 1), NT, 0, ctx->stream>>>(
+          S.U, S.P, ctx->partials, ctx->ctrl, ctx->L, 0, 0, kid<T>(KID_DELTA), ctx->grid64.spt);
+      CKL();
+      k_unpack_antiherm<double><<<grid1(V, NT), NT, 0, ctx->stream>>>(S.P, dst, V);
+      CKL();
+    }
   } else {
+    k_aos_to_planes<T><<<grid1(4 * V, NT), NT, 0, ctx->stream>>>(src, S.U, V, 4, LinkStore<T>::planes, 0, 4 * V);
+    CKL();
     TRY(launch_delta<T>(ctx, S, 0, 0));
     TRY(unpack_field<T>(ctx, S, dst));
   }

@@ -246,6 +246,40 @@ template <bool NEG> __device__ __forceinline__ void accumulate_link_q(const m3<d
 __device__ __forceinline__ double widen_exact(float v) { return widen_bits(v); }
 __device__ __forceinline__ double widen_exact(double v) { return v; }
 
+// The double Delta of one site: the six off-diagonal numbers and the first two of the diagonal in d, the site's
+// terms of theta and F in ts and fs. load(mu, site, u) reads a link.
+template <typename Load>
+__device__ __forceinline__ void delta_site(const Lattice &L, int64_t s, Load load, double d[8], double &ts, double &fs) {
+  int c[4];
+  site_coords(L, s, c);
+  long long acc[9];
+#pragma unroll
+  for (int e = 0; e < 9; ++e) acc[e] = 0;
+  bool bad = false;
+  fs = 0;
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    m3<double> u;
+    load(mu, site_back(L, s, mu, c[mu]), u);  // U_mu(x - mu)
+    accumulate_link_q<false>(u, acc, bad);
+    load(mu, s, u);  // - U_mu(x)
+    accumulate_link_q<true>(u, acc, bad);
+    fs += u.e[0].r + u.e[4].r + u.e[8].r;  // Re Tr U_mu(x)
+  }
+  constexpr double sc = 0x1p-56;
+#pragma unroll
+  for (int e = 0; e < 6; ++e) d[e] = __ll2double_rn(acc[e]) * sc;
+  // Delta_ii = 2i (Im B_ii - mean) = 2i (3 Im B_ii - sum) / 3
+  const long long sd = acc[6] + acc[7] + acc[8];
+  constexpr double w = 2.0 / 3.0 * sc;
+  d[6] = __ll2double_rn(3 * acc[6] - sd) * w;
+  d[7] = __ll2double_rn(3 * acc[7] - sd) * w;
+  const double a2 = __ll2double_rn(3 * acc[8] - sd) * w;
+  ts = d[6] * d[6] + d[7] * d[7] + a2 * a2 +
+       2 * (d[0] * d[0] + d[1] * d[1] + d[2] * d[2] + d[3] * d[3] + d[4] * d[4] + d[5] * d[5]);
+  if (bad) ts = __longlong_as_double(0x7FF8000000000000ll);  // non-finite or out-of-range link entries
+}
+
 // PT is the type of the packed output (T, or float when a double stage feeds a float FFT).
 template <typename T, int NT, typename PT = T>
 __device__ __forceinline__ void delta_body(const T *__restrict__ U, PT *__restrict__ P, double *partials, Ctrl *ctrl,
@@ -266,41 +300,16 @@ __device__ __forceinline__ void delta_body(const T *__restrict__ U, PT *__restri
     for (int k = 0; k < spt; ++k) {
       const int64_t s = ((int64_t)blockIdx.x * spt + k) * NT + threadIdx.x;
       if (s >= V) break;
-      int c[4];
-      site_coords(L, s, c);
-      long long acc[9];
-#pragma unroll
-      for (int e = 0; e < 9; ++e) acc[e] = 0;
-      bool bad = false;
-      double fs = 0;
-#pragma unroll
-      for (int mu = 0; mu < 4; ++mu) {
-        const double *plane = U + (int64_t)mu * link_plane_stride<T>(V);
-        m3<double> u;
-        load_link(plane, V, site_back(L, s, mu, c[mu]), u);  // U_mu(x - mu)
-        accumulate_link_q<false>(u, acc, bad);
-        load_link(plane, V, s, u);  // - U_mu(x)
-        accumulate_link_q<true>(u, acc, bad);
-        fs += u.e[0].r + u.e[4].r + u.e[8].r;  // Re Tr U_mu(x)
-      }
-      constexpr double sc = 0x1p-56;
-      double d[6];
-#pragma unroll
-      for (int e = 0; e < 6; ++e) d[e] = __ll2double_rn(acc[e]) * sc;
-      // Delta_ii = 2i (Im B_ii - mean) = 2i (3 Im B_ii - sum) / 3
-      const long long sd = acc[6] + acc[7] + acc[8];
-      constexpr double w = 2.0 / 3.0 * sc;
-      const double a0 = __ll2double_rn(3 * acc[6] - sd) * w, a1 = __ll2double_rn(3 * acc[7] - sd) * w;
-      const double a2 = __ll2double_rn(3 * acc[8] - sd) * w;
-      double ts = a0 * a0 + a1 * a1 + a2 * a2 +
-                  2 * (d[0] * d[0] + d[1] * d[1] + d[2] * d[2] + d[3] * d[3] + d[4] * d[4] + d[5] * d[5]);
-      if (bad) ts = __longlong_as_double(0x7FF8000000000000ll);  // non-finite or out-of-range link entries
+      double d[8], ts, fs;
+      delta_site(L, s, [&](int mu, int64_t at, m3<double> &u) {
+        load_link(U + (int64_t)mu * link_plane_stride<T>(V), V, at, u);
+      }, d, ts, fs);
       th += ts;
       f += fs;
       st(P, s, mkc(convert<PT>(d[0]), convert<PT>(d[1])));
       st(P, V + s, mkc(convert<PT>(d[2]), convert<PT>(d[3])));
       st(P, 2 * V + s, mkc(convert<PT>(d[4]), convert<PT>(d[5])));
-      st(P, 3 * V + s, mkc(convert<PT>(a0), convert<PT>(a1)));
+      st(P, 3 * V + s, mkc(convert<PT>(d[6]), convert<PT>(d[7])));
     }
   } else {
 #pragma unroll 1
@@ -433,6 +442,50 @@ __global__ void __launch_bounds__(NT, 5) k_delta_f32_tw(const float *__restrict_
     }
   }
   reduce_and_finalize_at<NT>(th, f, partials, ctrl, V, counts_update, 0.0, blockIdx.x + gridDim.x * blockIdx.y, nblk);
+}
+
+// Delta itself in double from the caller's links to the caller's matrices (both arrays of structures), without
+// the planes between: 720 bytes a site instead of 2100. A warp's 32 matrices leave through shared memory, so
+// that their stores are contiguous. Bound by the latency of its strided 16-byte loads: at 40^3 x 20 a call takes
+// 0.35 ms (0.37 with two resident blocks per SM, 0.40 with four), 0.68 with the planes, 0.14 by its bytes.
+template <int NT>
+__global__ void __launch_bounds__(NT, 3) k_delta_matrices(const double *__restrict__ U, double *__restrict__ D,
+                                                      double *partials, Ctrl *ctrl, Lattice L, int spt) {
+  __shared__ double2 rec[NT * 9];
+  const int64_t V = L.V;
+  const int lane = threadIdx.x & 31;
+  double2 *mine = rec + (threadIdx.x - lane) * 9;
+  double th = 0.0, f = 0.0;
+#pragma unroll 1
+  for (int k = 0; k < spt; ++k) {
+    const int64_t s = ((int64_t)blockIdx.x * spt + k) * NT + threadIdx.x, first = s - lane;
+    if (first >= V) break;
+    const int cnt = (int)min((int64_t)32, V - first);
+    if (lane < cnt) {
+      double d[8], ts, fs;
+      delta_site(L, s, [&](int mu, int64_t at, m3<double> &u) {
+#pragma unroll
+        for (int e = 0; e < 9; ++e) u.e[e] = ldg(U, ((int64_t)mu * V + at) * 9 + e);
+      }, d, ts, fs);
+      th += ts;
+      f += fs;
+      double2 *r = mine + lane * 9;
+      r[0] = make_double2(0.0, d[6]);
+      r[4] = make_double2(0.0, d[7]);
+      r[8] = make_double2(0.0, -(d[6] + d[7]));
+      r[1] = make_double2(d[0], d[1]);
+      r[2] = make_double2(d[2], d[3]);
+      r[5] = make_double2(d[4], d[5]);
+      r[3] = make_double2(-d[0], d[1]);
+      r[6] = make_double2(-d[2], d[3]);
+      r[7] = make_double2(-d[4], d[5]);
+    }
+    __syncwarp();
+    double2 *dst = reinterpret_cast<double2 *>(D) + first * 9;
+    for (int q = lane; q < cnt * 9; q += 32) dst[q] = mine[q];
+    __syncwarp();
+  }
+  reduce_and_finalize<NT>(th, f, partials, ctrl, V, 0);
 }
 
 // Rebuild the full anti-Hermitian traceless matrix from the packed fields (type PT), scaled by a.
@@ -793,7 +846,7 @@ __device__ __forceinline__ void update_links_general(double *U, const double *G,
 
 // Double links: general steps may be split between the FP64 pipe (the first fp64_even or fp64_odd directions
 // of a site, in even or odd warps) and the integer pipe (the others, in Q60); both forms are exact to FP64
-// rounding. All four in Q60 is the fastest: at 24^3 x 48 a general update takes 0.44 ms, against 0.46 with
+// rounding. All four in Q60 is the fastest: at 24^3 x 48 a general update takes 0.41 ms, against 0.46 with
 // one direction in every other warp in FP64, 0.49 with two in every warp and 0.57 with two in the 61-bit form
 // of q61.cuh, which joins and splits the limbs at every product. The integer and conversion instructions
 // bound it (16 warps per SM, the bytes would take 0.13 ms).
