@@ -257,6 +257,7 @@ template <typename T>
 __global__ void __launch_bounds__(512) k_fft_pass(T *__restrict__ data, int64_t V, const __grid_constant__ PassDesc pd,
                                                  const __grid_constant__ FFTTables tb, const Ctrl *ctrl,
                                                  int check_active, int tkid) {
+  follow_on();
   data += (int64_t)blockIdx.z * 4 * V * 2;
   ctrl += blockIdx.z;
   if (!should_run<T>(ctrl, check_active)) return;
@@ -283,7 +284,7 @@ __global__ void __launch_bounds__(512) k_fft_pass(T *__restrict__ data, int64_t 
     for (int e = threadIdx.x; e < pd.rows * (int)pd.dnx.d; e += blockDim.x) {
       const unsigned r = div_by(e, pd.dnx), x = e - r * pd.dnx.d;
       V2 v = {};
-      if (e < nel) v = __ldg(field + base + e);
+      if (e < nel) v = ldv(field + base + e);
       tile[r * pd.pitch + x] = from_vec<T>(v);
     }
   } else {
@@ -293,7 +294,7 @@ __global__ void __launch_bounds__(512) k_fft_pass(T *__restrict__ data, int64_t 
 #pragma unroll 4
     for (int r = row0; r < pd.rows; r += rstep) {
       V2 v = {};
-      if (r < rows) v = __ldg(field + base + r * pd.rstride);
+      if (r < rows) v = ldv(field + base + r * pd.rstride);
       tile[r * pd.pitch + c] = from_vec<T>(v);
     }
   }

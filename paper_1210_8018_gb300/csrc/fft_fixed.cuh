@@ -96,6 +96,7 @@ template <typename T, int N> __device__ __forceinline__ void load_twiddles(cx<T>
 template <typename T, int NX, int NY, bool INV, int NT>
 __global__ void __launch_bounds__(NT) k_fx_plane(T *__restrict__ data, int64_t V, FFTTables tb, const Ctrl *ctrl,
                                                 int check_active, int tkid, int ntiles) {
+  follow_on();
   (void)ntiles;
   data += (int64_t)blockIdx.z * 4 * V * 2;
   ctrl += blockIdx.z;
@@ -116,7 +117,7 @@ __global__ void __launch_bounds__(NT) k_fx_plane(T *__restrict__ data, int64_t V
   for (int k = 0; k < PER; ++k) {
     const int e = threadIdx.x + k * NT;
     if (e < NEL) {
-      reg[k] = from_vec<T>(__ldg(reinterpret_cast<const typename vec2<T>::type *>(src) + e));
+      reg[k] = from_vec<T>(ldv(reinterpret_cast<const typename vec2<T>::type *>(src) + e));
     }
   }
 #pragma unroll
@@ -161,6 +162,7 @@ template <typename T, int N, int C, int MODE, int NT, int FPB = 4>
 __global__ void __launch_bounds__(NT) k_fx_cols(T *__restrict__ data, int64_t V, int64_t rstride, int ncb,
                                                int64_t ostride, FFTTables tb, const Ctrl *ctrl, int check_active,
                                                int tkid, int twmu, int ntiles) {
+  follow_on();
   if constexpr (prefetch_tiles<T, 2, MODE>()) {
   data += (int64_t)blockIdx.z * 4 * V * 2;
   ctrl += blockIdx.z;
@@ -192,7 +194,7 @@ __global__ void __launch_bounds__(NT) k_fx_cols(T *__restrict__ data, int64_t V,
 #pragma unroll
       for (int k = 0; k < PER; ++k) {
         const int e = threadIdx.x + k * NT;
-        if (e < NEL) reg[f][k] = __ldg(src + base + (e / C) * rstride + (e % C));
+        if (e < NEL) reg[f][k] = ldv(src + base + (e / C) * rstride + (e % C));
       }
     }
   };
@@ -284,7 +286,7 @@ __global__ void __launch_bounds__(NT) k_fx_cols(T *__restrict__ data, int64_t V,
       const int e = threadIdx.x + k * NT;
       if (e < NEL) {
         const int n = e / C, c = e % C;
-        reg[k] = from_vec<T>(__ldg(reinterpret_cast<const typename vec2<T>::type *>(src) + base + n * rstride + c));
+        reg[k] = from_vec<T>(ldv(reinterpret_cast<const typename vec2<T>::type *>(src) + base + n * rstride + c));
       }
     }
 #pragma unroll
@@ -360,6 +362,7 @@ __global__ void __launch_bounds__(NT) k_fx_cols(T *__restrict__ data, int64_t V,
 template <typename T, bool INV>
 __global__ void __launch_bounds__(512, 3) k_fx_plane64(T *__restrict__ data, int64_t V, FFTTables tb, const Ctrl *ctrl,
                                                       int check_active, int tkid, int ntiles) {
+  follow_on();
   constexpr int N = 64, R = 8, P = 72;
   static_assert(std::is_same<T, float>::value, "float pass");
   (void)ntiles;
@@ -378,7 +381,7 @@ __global__ void __launch_bounds__(512, 3) k_fx_plane64(T *__restrict__ data, int
   cx<T> v[R];
   if constexpr (!INV) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = from_vec<T>(__ldg(pl + y * N + j + R * r));
+    for (int r = 0; r < R; ++r) v[r] = from_vec<T>(ldv(pl + y * N + j + R * r));
     dft<T, R, false>(v);
 #pragma unroll
     for (int r = 1; r < R; ++r) v[r] = v[r] * twx[j * r];
@@ -406,7 +409,7 @@ __global__ void __launch_bounds__(512, 3) k_fx_plane64(T *__restrict__ data, int
     for (int r = 0; r < R; ++r) pl[(R * jy + r) * N + x] = to_vec<T>(v[r]);
   } else {
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = from_vec<T>(__ldg(pl + (R * jy + r) * N + x));
+    for (int r = 0; r < R; ++r) v[r] = from_vec<T>(ldv(pl + (R * jy + r) * N + x));
     dft<T, R, true>(v);
 #pragma unroll
     for (int r = 0; r < R; ++r) tile[at(R * jy + r, x)] = v[r];
@@ -454,6 +457,7 @@ template <typename T, int C, int NT>
 __global__ void __launch_bounds__(NT, 5) k_fx_tfilter64(T *__restrict__ data, int64_t V, int64_t rstride, int ncb,
                                                        int64_t ostride, FFTTables tb, const Ctrl *ctrl,
                                                        int check_active, int tkid, int twmu, int ntiles) {
+  follow_on();
   constexpr int N = 64, R = 8;
   static_assert(NT == C * R, "eight threads per column");
   static_assert(std::is_same<T, float>::value, "float pass");
@@ -473,7 +477,7 @@ __global__ void __launch_bounds__(NT, 5) k_fx_tfilter64(T *__restrict__ data, in
   auto fetch = [&](int bb) {
     const int64_t base = base_of(bb);
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = from_vec<T>(__ldg(fld + base + (int64_t)(j + R * r) * rstride));
+    for (int r = 0; r < R; ++r) v[r] = from_vec<T>(ldv(fld + base + (int64_t)(j + R * r) * rstride));
   };
   if (threadIdx.x < N) srow[threadIdx.x] = convert<T>(__ldg(tb.p2part[3] + threadIdx.x));
   const cx<T> *tw = reinterpret_cast<const cx<T> *>(tb.tw[twmu]);

@@ -159,6 +159,7 @@ struct lgf_ctx {
   int64_t twalk_min_blocks = 2048;  // LGF_TWALK_MIN_BLOCKS
   int handover_split[2] = {2, 2};  // links per site in FP64 (even, odd warps), the rest in fixed point
   int update_split[2] = {0, 0};    // the same for the general (large-step) form of the double update
+  bool pdl = true;             // kernels of the iteration launched behind one another (LGF_PDL=0: off)
   bool reunit_fp64 = false;    // float stages: periodic projection onto SU(3) in double instead of float
   bool resid_base_ready = false;  // the float link planes hold the double links rounded (by the handover)
   double resid_theta0 = 0;  // theta of the residual stage's base links
@@ -206,11 +207,37 @@ lgf_status fail(lgf_ctx *c, lgf_status st, const std::string &msg) {
     if (e_ != cudaSuccess) return fail(ctx, LGF_ECUDA, std::string("kernel launch: ") + cudaGetErrorString(e_)); \
   } while (0)
 
-#define TRY(x)                   \
+#define TRY(...)                 \
   do {                           \
-    lgf_status s_ = (x);         \
+    lgf_status s_ = (__VA_ARGS__); \
     if (s_ != LGF_OK) return s_; \
   } while (0)
+
+// Launch of a kernel of the iteration whose first statement is follow_on(): an iteration is seven to nine
+// kernels, and on small lattices the gaps between them cost as much as the kernels. Fix at 8^4 1.80 -> 1.27 ms,
+// 16^3 x 32 3.50 -> 2.83, 18x12x10x15 (double) 3.89 -> 3.38, 32^4 14.8 -> 14.0, 64^4 191.2 -> 190.1.
+lgf_status launch_next_ptr(lgf_ctx *ctx, const void *k, dim3 grid, unsigned threads, size_t smem, void **args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = ctx->stream;
+  cudaLaunchAttribute a = {};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &a;
+  c.numAttrs = ctx->pdl ? 1 : 0;
+  CK(cudaLaunchKernelExC(&c, k, args));
+  return LGF_OK;
+}
+template <typename... P, typename... A>
+lgf_status launch_next(lgf_ctx *ctx, void (*k)(P...), dim3 grid, unsigned threads, size_t smem, A... args) {
+  static_assert(sizeof...(P) == sizeof...(A), "arguments");
+  return [&](P... p) {
+    void *ptrs[] = {(void *)&p...};
+    return launch_next_ptr(ctx, (const void *)k, grid, threads, smem, ptrs);
+  }(args...);
+}
 
 unsigned grid1(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
@@ -726,16 +753,15 @@ template <typename T> lgf_status launch_delta(lgf_ctx *ctx, State<T> &S, int cou
     FT *P = reinterpret_cast<FT *>(S.P);
     if constexpr (std::is_same<T, float>::value) {
       if (twalk_on(ctx))
-        k_delta_f32_tw<NT, kTwalkSlices><<<twalk_grid(ctx), NT, 0, ctx->stream>>>(
-            S.U, P, ctx->partials, ctx->ctrl, ctx->L, counts_update, check_active, kid<T>(KID_DELTA));
+        TRY(launch_next(ctx, k_delta_f32_tw<NT, kTwalkSlices>, twalk_grid(ctx), NT, 0, S.U, P, ctx->partials,
+                        ctx->ctrl, ctx->L, counts_update, check_active, kid<T>(KID_DELTA)));
       else
-        k_delta_f32<NT><<<dim3(ctx->grid32.blocks, 1, ctx->nb), NT, 0, ctx->stream>>>(S.U, P, ctx->partials, ctx->ctrl, ctx->L, counts_update,
-                                                      check_active, kid<T>(KID_DELTA), ctx->grid32.spt);
+        TRY(launch_next(ctx, k_delta_f32<NT>, dim3(ctx->grid32.blocks, 1, ctx->nb), NT, 0, S.U, P, ctx->partials,
+                        ctx->ctrl, ctx->L, counts_update, check_active, kid<T>(KID_DELTA), ctx->grid32.spt));
     }
     else
-      k_delta<T, NT, FT><<<dim3(ctx->grid64.blocks, 1, ctx->nb), NT, 0, ctx->stream>>>(S.U, P, ctx->partials, ctx->ctrl, ctx->L, counts_update,
-                                                       check_active, kid<T>(KID_DELTA), ctx->grid64.spt);
-    CKL();
+      TRY(launch_next(ctx, k_delta<T, NT, FT>, dim3(ctx->grid64.blocks, 1, ctx->nb), NT, 0, S.U, P, ctx->partials,
+                      ctx->ctrl, ctx->L, counts_update, check_active, kid<T>(KID_DELTA), ctx->grid64.spt));
     return LGF_OK;
   }));
   return timed_end(ctx);
@@ -755,7 +781,7 @@ template <typename T> lgf_status launch_filter(lgf_ctx *ctx, State<T> &S, T *dat
       FFTTables tb = S.tables;
       const Ctrl *c = ctx->ctrl;
       void *args[] = {&data, &V, &pd, &tb, &c, &check_active, (void *)&tk};
-      CK(cudaLaunchKernel(fft_generic_kernel<FT>(), grid, dim3(p.threads), args, p.smem, ctx->stream));
+      TRY(launch_next_ptr(ctx, fft_generic_kernel<FT>(), grid, p.threads, p.smem, args));
     } else if (p.kind == 1 || p.kind == 4) {
       dim3 grid(p.grid_x > 0 ? p.grid_x : p.nblocks, 4, ctx->nb);
       int64_t V = ctx->V;
@@ -763,7 +789,7 @@ template <typename T> lgf_status launch_filter(lgf_ctx *ctx, State<T> &S, T *dat
       const Ctrl *c = ctx->ctrl;
       int nt = p.nblocks;
       void *args[] = {&data, &V, &tb, &c, &check_active, (void *)&tk, &nt};
-      CK(cudaLaunchKernel(fixed_kernel<FT>(p), grid, dim3(p.threads), args, p.smem, ctx->stream));
+      TRY(launch_next_ptr(ctx, fixed_kernel<FT>(p), grid, p.threads, p.smem, args));
     } else {
       dim3 grid(p.grid_x > 0 ? p.grid_x : p.nblocks, p.mode == 2 ? 4 / filter_fields_per_block<FT>() : 4, ctx->nb);
       int64_t V = ctx->V, rs = p.rstride, os = p.ostride;
@@ -771,7 +797,7 @@ template <typename T> lgf_status launch_filter(lgf_ctx *ctx, State<T> &S, T *dat
       FFTTables tb = S.tables;
       const Ctrl *c = ctx->ctrl;
       void *args[] = {&data, &V, &rs, &ncb, &os, &tb, &c, &check_active, (void *)&tk, &twmu, &nt};
-      CK(cudaLaunchKernel(fixed_kernel<FT>(p), grid, dim3(p.threads), args, p.smem, ctx->stream));
+      TRY(launch_next_ptr(ctx, fixed_kernel<FT>(p), grid, p.threads, p.smem, args));
     }
     CKL();
     TRY(timed_end(ctx));
@@ -784,10 +810,9 @@ template <typename T> lgf_status launch_gauge(lgf_ctx *ctx, State<T> &S, double 
   TRY(timed_begin(ctx, kid<T>(KID_GAUGE)));
   TRY(with_fft_type<T>(ctx, [&](auto tag) -> lgf_status {
     using FT = decltype(tag);
-    k_gauge<T, NT, FT><<<dim3(grid1(ctx->V, NT), 1, ctx->nb), NT, 0, ctx->stream>>>(
-        reinterpret_cast<const FT *>(S.P), S.G, S.A, (T)(0.5 * alpha), ctx->V, ctx->ctrl, check_active, kid<T>(KID_GAUGE),
-        ctx->small_step ? 1 : 0);
-    CKL();
+    TRY(launch_next(ctx, k_gauge<T, NT, FT>, dim3(grid1(ctx->V, NT), 1, ctx->nb), NT, 0,
+                    reinterpret_cast<const FT *>(S.P), S.G, S.A, (T)(0.5 * alpha), ctx->V, ctx->ctrl, check_active,
+                    kid<T>(KID_GAUGE), ctx->small_step ? 1 : 0));
     return LGF_OK;
   }));
   return timed_end(ctx);
@@ -796,15 +821,13 @@ template <typename T> lgf_status launch_gauge(lgf_ctx *ctx, State<T> &S, double 
 template <typename T> lgf_status launch_update(lgf_ctx *ctx, State<T> &S, int check_active) {
   TRY(timed_begin(ctx, kid<T>(KID_UPDATE)));
   if constexpr (std::is_same<T, double>::value) {
-    k_update<double, NT_UPDATE64><<<dim3(grid1(ctx->V, NT_UPDATE64), 1, ctx->nb), NT_UPDATE64,
-                                    update_smem_bytes<NT_UPDATE64>(), ctx->stream>>>(
-        S.U, S.G, S.A, ctx->L, ctx->ctrl, check_active, kid<T>(KID_UPDATE), ctx->small_step ? 1 : 0,
-        ctx->update_split[0], ctx->update_split[1]);
+    TRY(launch_next(ctx, k_update<double, NT_UPDATE64>, dim3(grid1(ctx->V, NT_UPDATE64), 1, ctx->nb), NT_UPDATE64,
+                    update_smem_bytes<NT_UPDATE64>(), S.U, S.G, S.A, ctx->L, ctx->ctrl, check_active,
+                    kid<T>(KID_UPDATE), ctx->small_step ? 1 : 0, ctx->update_split[0], ctx->update_split[1]));
   } else {
-    k_update<T, NT><<<dim3(grid1(ctx->V, NT), 1, ctx->nb), NT, 0, ctx->stream>>>(S.U, S.G, nullptr, ctx->L, ctx->ctrl,
-                                                                               check_active, kid<T>(KID_UPDATE), 0, 0, 0);
+    TRY(launch_next(ctx, k_update<T, NT>, dim3(grid1(ctx->V, NT), 1, ctx->nb), NT, 0, S.U, S.G, nullptr, ctx->L,
+                    ctx->ctrl, check_active, kid<T>(KID_UPDATE), 0, 0, 0));
   }
-  CKL();
   return timed_end(ctx);
 }
 
@@ -820,19 +843,16 @@ template <typename T> lgf_status launch_iteration(lgf_ctx *ctx, State<T> &S, dou
 // packed in float, float FFT passes, g formed in double from the float Delta-tilde, double update.
 lgf_status launch_delta_d2f(lgf_ctx *ctx, int counts_update, int check_active) {
   TRY(timed_begin(ctx, kid<double>(KID_DELTA)));
-  k_delta<double, NT, float><<<dim3(ctx->grid64.blocks, 1, ctx->nb), NT, 0, ctx->stream>>>(
-      ctx->s64.U, ctx->s32.P, ctx->partials, ctx->ctrl, ctx->L, counts_update, check_active, kid<double>(KID_DELTA),
-      ctx->grid64.spt);
-  CKL();
+  TRY(launch_next(ctx, k_delta<double, NT, float>, dim3(ctx->grid64.blocks, 1, ctx->nb), NT, 0, ctx->s64.U,
+                  ctx->s32.P, ctx->partials, ctx->ctrl, ctx->L, counts_update, check_active, kid<double>(KID_DELTA),
+                  ctx->grid64.spt));
   return timed_end(ctx);
 }
 lgf_status launch_iteration_fft32(lgf_ctx *ctx, double alpha) {
   TRY(launch_filter<float>(ctx, ctx->s32, ctx->s32.P, 2));
   TRY(timed_begin(ctx, kid<double>(KID_GAUGE)));
-  k_gauge<double, NT, float><<<dim3(grid1(ctx->V, NT), 1, ctx->nb), NT, 0, ctx->stream>>>(
-      ctx->s32.P, ctx->s64.G, ctx->s64.A, 0.5 * alpha, ctx->V, ctx->ctrl, 1, kid<double>(KID_GAUGE),
-      ctx->small_step ? 1 : 0);
-  CKL();
+  TRY(launch_next(ctx, k_gauge<double, NT, float>, dim3(grid1(ctx->V, NT), 1, ctx->nb), NT, 0, ctx->s32.P, ctx->s64.G,
+                  ctx->s64.A, 0.5 * alpha, ctx->V, ctx->ctrl, 1, kid<double>(KID_GAUGE), ctx->small_step ? 1 : 0));
   TRY(timed_end(ctx));
   TRY(launch_update<double>(ctx, ctx->s64, 1));
   return launch_delta_d2f(ctx, 1, 1);
@@ -850,21 +870,20 @@ lgf_status launch_iteration_float(lgf_ctx *ctx, double alpha, bool reunit) {
   if (twalk_on(ctx)) {
     constexpr int TCH = kTwalkSlices;
     if (reunit && ctx->reunit_fp64)
-      k_update_fused_f32_tw<NT, 2, TCH><<<twalk_grid(ctx), NT, 0, ctx->stream>>>(S.U, S.P, ctx->Gacc, ha, ctx->L,
-                                                                                 ctx->ctrl, kidx);
+      TRY(launch_next(ctx, k_update_fused_f32_tw<NT, 2, TCH>, twalk_grid(ctx), NT, 0, S.U, S.P, ctx->Gacc, ha, ctx->L,
+                      ctx->ctrl, kidx));
     else if (reunit)
-      k_update_fused_f32_tw<NT, 1, TCH><<<twalk_grid(ctx), NT, 0, ctx->stream>>>(S.U, S.P, ctx->Gacc, ha, ctx->L,
-                                                                                 ctx->ctrl, kidx);
+      TRY(launch_next(ctx, k_update_fused_f32_tw<NT, 1, TCH>, twalk_grid(ctx), NT, 0, S.U, S.P, ctx->Gacc, ha, ctx->L,
+                      ctx->ctrl, kidx));
     else
-      k_update_fused_f32_tw<NT, 0, TCH><<<twalk_grid(ctx), NT, 0, ctx->stream>>>(S.U, S.P, ctx->Gacc, ha, ctx->L,
-                                                                                 ctx->ctrl, kidx);
+      TRY(launch_next(ctx, k_update_fused_f32_tw<NT, 0, TCH>, twalk_grid(ctx), NT, 0, S.U, S.P, ctx->Gacc, ha, ctx->L,
+                      ctx->ctrl, kidx));
   } else if (reunit && ctx->reunit_fp64)
-    k_update_fused_f32<NT, 2><<<grid, NT, 0, ctx->stream>>>(S.U, S.P, ctx->Gacc, ha, ctx->L, ctx->ctrl, kidx);
+    TRY(launch_next(ctx, k_update_fused_f32<NT, 2>, grid, NT, 0, S.U, S.P, ctx->Gacc, ha, ctx->L, ctx->ctrl, kidx));
   else if (reunit)
-    k_update_fused_f32<NT, 1><<<grid, NT, 0, ctx->stream>>>(S.U, S.P, ctx->Gacc, ha, ctx->L, ctx->ctrl, kidx);
+    TRY(launch_next(ctx, k_update_fused_f32<NT, 1>, grid, NT, 0, S.U, S.P, ctx->Gacc, ha, ctx->L, ctx->ctrl, kidx));
   else
-    k_update_fused_f32<NT, 0><<<grid, NT, 0, ctx->stream>>>(S.U, S.P, ctx->Gacc, ha, ctx->L, ctx->ctrl, kidx);
-  CKL();
+    TRY(launch_next(ctx, k_update_fused_f32<NT, 0>, grid, NT, 0, S.U, S.P, ctx->Gacc, ha, ctx->L, ctx->ctrl, kidx));
   TRY(timed_end(ctx));
   return launch_delta<float>(ctx, S, 1, 1);
 }
@@ -917,14 +936,13 @@ lgf_status launch_delta_residual(lgf_ctx *ctx, int counts_update) {
   TRY(with_fft_type<double>(ctx, [&](auto tag) -> lgf_status {
     using FT = decltype(tag);
     if (twalk_on(ctx))
-      k_delta_residual_tw<NT, FT, kTwalkSlices><<<twalk_grid(ctx), NT, 0, ctx->stream>>>(
-          ctx->Rres, reinterpret_cast<const FT *>(ctx->s64.P), ctx->s32.P, ctx->partials, ctx->ctrl, ctx->L,
-          counts_update, kid<float>(KID_DELTA_RESIDUAL));
+      TRY(launch_next(ctx, k_delta_residual_tw<NT, FT, kTwalkSlices>, twalk_grid(ctx), NT, 0, ctx->Rres,
+                      reinterpret_cast<const FT *>(ctx->s64.P), ctx->s32.P, ctx->partials, ctx->ctrl, ctx->L,
+                      counts_update, kid<float>(KID_DELTA_RESIDUAL)));
     else
-      k_delta_residual<NT, FT><<<dim3(ctx->grid_resid.blocks, 1, ctx->nb), NT, 0, ctx->stream>>>(
-          ctx->Rres, reinterpret_cast<const FT *>(ctx->s64.P), ctx->s32.P, ctx->partials, ctx->ctrl, ctx->L,
-          counts_update, kid<float>(KID_DELTA_RESIDUAL), ctx->grid_resid.spt);
-    CKL();
+      TRY(launch_next(ctx, k_delta_residual<NT, FT>, dim3(ctx->grid_resid.blocks, 1, ctx->nb), NT, 0, ctx->Rres,
+                      reinterpret_cast<const FT *>(ctx->s64.P), ctx->s32.P, ctx->partials, ctx->ctrl, ctx->L,
+                      counts_update, kid<float>(KID_DELTA_RESIDUAL), ctx->grid_resid.spt));
     return LGF_OK;
   }));
   return timed_end(ctx);
@@ -960,14 +978,11 @@ lgf_status launch_iteration_residual(lgf_ctx *ctx, double alpha) {
   TRY(launch_filter<float>(ctx, ctx->s32, ctx->s32.P, 3));
   TRY(timed_begin(ctx, kid<float>(KID_UPDATE_RESIDUAL)));
   if (twalk_on(ctx))
-    k_update_residual_tw<NT, kTwalkSlices><<<twalk_grid(ctx), NT, 0, ctx->stream>>>(
-        ctx->s32.U, ctx->Rres, ctx->Kres, ctx->s32.P, (float)(0.5 * alpha), ctx->L, ctx->ctrl,
-        kid<float>(KID_UPDATE_RESIDUAL));
+    TRY(launch_next(ctx, k_update_residual_tw<NT, kTwalkSlices>, twalk_grid(ctx), NT, 0, ctx->s32.U, ctx->Rres,
+                    ctx->Kres, ctx->s32.P, (float)(0.5 * alpha), ctx->L, ctx->ctrl, kid<float>(KID_UPDATE_RESIDUAL)));
   else
-    k_update_residual<NT><<<dim3(grid1(ctx->V, NT), 1, ctx->nb), NT, 0, ctx->stream>>>(
-        ctx->s32.U, ctx->Rres, ctx->Kres, ctx->s32.P, (float)(0.5 * alpha), ctx->L, ctx->ctrl,
-        kid<float>(KID_UPDATE_RESIDUAL));
-  CKL();
+    TRY(launch_next(ctx, k_update_residual<NT>, dim3(grid1(ctx->V, NT), 1, ctx->nb), NT, 0, ctx->s32.U, ctx->Rres,
+                    ctx->Kres, ctx->s32.P, (float)(0.5 * alpha), ctx->L, ctx->ctrl, kid<float>(KID_UPDATE_RESIDUAL)));
   TRY(timed_end(ctx));
   return launch_delta_residual(ctx, 1);
 }
@@ -1224,6 +1239,8 @@ static lgf_status create_ctx(const int n[4], int nb, lgf_ctx **out) {
       ctx->update_split[0] = us[0] - '0';
       ctx->update_split[1] = us[1] - '0';
     }
+    const char *pd = std::getenv("LGF_PDL");
+    ctx->pdl = !(pd && pd[0] == '0');
     const char *rf = std::getenv("LGF_REUNIT_FP64");
     ctx->reunit_fp64 = rf && rf[0] == '1';
   }

@@ -39,6 +39,7 @@ template <int NT, int REUNIT>
 __global__ void __launch_bounds__(NT) k_update_fused_f32(float *__restrict__ U, const float *__restrict__ P,
                                                         float *__restrict__ Gacc, float half_alpha, Lattice L,
                                                         const Ctrl *ctrl, int tkid) {
+  follow_on();
   const int64_t V = L.V;
   {
     const int cfg = blockIdx.z;
@@ -88,6 +89,7 @@ template <int NT, int REUNIT, int TCH>
 __global__ void __launch_bounds__(NT) k_update_fused_f32_tw(float *__restrict__ U, const float *__restrict__ P,
                                                            float *__restrict__ Gacc, float half_alpha, Lattice L,
                                                            const Ctrl *ctrl, int tkid) {
+  follow_on();
   const int64_t V = L.V;
   {
     const int cfg = blockIdx.z;
@@ -348,6 +350,7 @@ template <int NT, typename PT>
 __global__ void __launch_bounds__(NT, 4) k_delta_residual(const float *__restrict__ R, const PT *__restrict__ Ph,
                                                       float *__restrict__ P, double *partials, Ctrl *ctrl, Lattice L,
                                                       int counts_update, int tkid, int spt) {
+  follow_on();
   const int64_t V = L.V;
   {
     const int cfg = blockIdx.z;
@@ -407,6 +410,7 @@ template <int NT, typename PT, int TCH>
 __global__ void __launch_bounds__(NT, 4) k_delta_residual_tw(const float *__restrict__ R, const PT *__restrict__ Ph,
                                                          float *__restrict__ P, double *partials, Ctrl *ctrl,
                                                          Lattice L, int counts_update, int tkid) {
+  follow_on();
   const int64_t V = L.V;
   const unsigned nblk = gridDim.x * gridDim.y;
   {
@@ -522,6 +526,7 @@ template <int NT>
 __global__ void __launch_bounds__(NT) k_update_residual(const float *__restrict__ B, float *__restrict__ R,
                                                        float *__restrict__ K, const float *__restrict__ P,
                                                        float half_alpha, Lattice L, const Ctrl *ctrl, int tkid) {
+  follow_on();
   const int64_t V = L.V;
   {
     const int cfg = blockIdx.z;
@@ -573,6 +578,7 @@ template <int NT, int TCH>
 __global__ void __launch_bounds__(NT, 2) k_update_residual_tw(const float *__restrict__ B, float *__restrict__ R,
                                                           float *__restrict__ K, const float *__restrict__ P,
                                                           float half_alpha, Lattice L, const Ctrl *ctrl, int tkid) {
+  follow_on();
   const int64_t V = L.V;
   {
     const int cfg = blockIdx.z;

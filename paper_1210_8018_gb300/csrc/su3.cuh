@@ -58,12 +58,36 @@ template <typename T> __device__ __forceinline__ typename vec2<T>::type to_vec(c
 }
 template <> __device__ __forceinline__ float4 to_vec<df64>(cx<df64> a) { return make_float4(a.r.hi, a.r.lo, a.i.hi, a.i.lo); }
 
-// Read-only global load / store of one complex element (base counts real components of type T).
+// Global load of a vector in the order of the program: fields that another kernel of the iteration may have
+// written after this one was placed on the chip (follow_on) are not read-only for its lifetime, which the
+// non-coherent __ldg takes for granted, and nothing moves a volatile load to before the wait.
+__device__ __forceinline__ float2 ldv(const float2 *p) {
+  float2 v;
+  asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double2 ldv(const double2 *p) {
+  double2 v;
+  asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 ldv(const float4 *p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ int4 ldv(const int4 *p) {
+  int4 v;
+  asm volatile("ld.global.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+
+// Global load / store of one complex element (base counts real components of type T).
 template <typename T> __device__ __forceinline__ cx<T> ldg(const T *base, int64_t idx) {
-  return from_vec<T>(__ldg(reinterpret_cast<const typename vec2<T>::type *>(base) + idx));
+  return from_vec<T>(ldv(reinterpret_cast<const typename vec2<T>::type *>(base) + idx));
 }
 template <typename T> __device__ __forceinline__ cx<T> ld(const T *base, int64_t idx) {
-  return from_vec<T>(reinterpret_cast<const typename vec2<T>::type *>(base)[idx]);
+  return from_vec<T>(ldv(reinterpret_cast<const typename vec2<T>::type *>(base) + idx));
 }
 template <typename T> __device__ __forceinline__ void st(T *base, int64_t idx, cx<T> a) {
   reinterpret_cast<typename vec2<T>::type *>(base)[idx] = to_vec<T>(a);
