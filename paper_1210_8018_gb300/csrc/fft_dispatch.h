@@ -13,6 +13,15 @@ namespace lgf {
 // kind 3 = the float column pass with the filter held in registers (k_fx_tfilter64: N = 64, C = 32, mode 2);
 // kind 4 = the float 64 x 64 xy plane pass held in registers (k_fx_plane64; mode 0 forward, 1 inverse).
 template <typename FT> const void *fft_fixed_kernel(int kind, int mode, int N, int C);
+// The float pass over z and t with the filter (k_fx_zt) for extents of the table, with its columns per block,
+// threads and shared memory.
+struct ZtKernel {
+  const void *kernel;
+  int C, threads;
+  size_t smem;
+};
+constexpr int kZtSites = 2048;  // largest Nz Nt that takes it
+ZtKernel fft_float_zt(int nz, int nt);
 // Generic pass (fft.cuh, k_fft_pass).
 template <typename FT> const void *fft_generic_kernel();
 

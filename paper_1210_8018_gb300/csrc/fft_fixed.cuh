@@ -531,4 +531,130 @@ __global__ void __launch_bounds__(NT, 5) k_fx_tfilter64(T *__restrict__ data, in
   }
 }
 
+// ---------------------------------------------------------------------------------------------
+// z and t together with the filter: a block takes the whole z and t extents of C columns of one packed field
+// through z forward, t forward, the filter, t inverse and z inverse in shared memory -- one pass over the field and
+// one launch where the column passes make three. The butterflies, their order and the weights are those of
+// k_fx_cols, and what it rounds when it stores a field is rounded here in the tile: the same bits.
+// Tile: element (t, z, c) at (t PZ + z + z / 8) C + c. Threads run through c, then j or the block of a z stage
+// (the padding after every eighth z keeps the last stage, which strides by its radix, free of bank conflicts), then
+// t; in the t stages through c, z, then the rest. The trips through shared memory bound it, which is why the
+// planner takes it up to Nz Nt = kZtSites only. Measured per iteration, with the events of the timing mode, against
+// the three column passes: 16 x 32 (16^3 x 32) 16 against 35 us, 32 x 32 (32^4) 44 / 68, 32 x 48 (48^2 x 32 x 48)
+// 155 / 181, 32 x 64 (64^2 x 32 x 64) 289 / 323; but 48 x 48 (48^4) 299 / 277, 64 x 64 (64^4) 621 / 572.
+// Mixed fix at 8^4 1.28 -> 1.15 ms, 16^3 x 32 2.82 -> 2.65, 32^4 14.0 -> 13.7.
+// ---------------------------------------------------------------------------------------------
+template <int NZ, int NTT> struct ZtTile {
+  // 64-byte runs in the small tiles, else 32-byte runs (32 x 32: 44 us against 48 with 64-byte runs at 32^4)
+  static constexpr int C = NZ * NTT <= 768 ? 8 : 4;
+  static constexpr int PZ = NZ + NZ / 8;
+  static constexpr int NEL = NZ * NTT * C;
+  static constexpr int threads = NEL >= 6144 ? 512 : 256;
+  static constexpr size_t smem = (size_t)(NTT * PZ * C + NZ + NTT) * 8 + (size_t)(NZ * C + NTT) * 4;
+  __device__ static __forceinline__ int at(int t, int z) { return (t * PZ + z + (z >> 3)) * C; }
+};
+template <typename T, int NZ, int NTT, bool ALONG_T, int L, int R, bool INV>
+__device__ __forceinline__ void zt_stage(cx<T> *tile, const cx<T> *tw) {
+  using Z = ZtTile<NZ, NTT>;
+  constexpr int C = Z::C, N = ALONG_T ? NTT : NZ, M = L / R, NB = N / R, TWSTEP = N / L, ITEMS = Z::NEL / R;
+#pragma unroll 2
+  for (int w = threadIdx.x; w < ITEMS; w += Z::threads) {
+    const int c = w % C, rest = w / C;
+    const int beta = ALONG_T ? rest / NZ : rest % NB, other = ALONG_T ? rest % NZ : rest / NB;
+    const int j = beta % M, n0 = (beta / M) * L + j;
+    cx<T> *p[R];
+    cx<T> v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      p[r] = tile + c + (ALONG_T ? Z::at(n0 + r * M, other) : Z::at(other, n0 + r * M));
+      v[r] = *p[r];
+    }
+    if constexpr (!INV) {
+      dft<T, R, false>(v);
+      if constexpr (M > 1) {
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[r] = v[r] * tw[j * r * TWSTEP];
+      }
+    } else {
+      if constexpr (M > 1) {
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[r] = v[r] * conjg(tw[j * r * TWSTEP]);
+      }
+      dft<T, R, true>(v);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) *p[r] = v[r];
+  }
+  __syncthreads();
+}
+template <typename T, int NZ, int NTT, bool ALONG_T, bool INV, int L, int R, int... Rest>
+__device__ __forceinline__ void zt_stages(cx<T> *tile, const cx<T> *tw) {
+  if constexpr (!INV) zt_stage<T, NZ, NTT, ALONG_T, L, R, false>(tile, tw);
+  if constexpr (sizeof...(Rest) > 0) zt_stages<T, NZ, NTT, ALONG_T, INV, L / R, Rest...>(tile, tw);
+  if constexpr (INV) zt_stage<T, NZ, NTT, ALONG_T, L, R, true>(tile, tw);
+}
+template <typename T, int NZ, int NTT, bool ALONG_T, bool INV, int... Rs>
+__device__ __forceinline__ void zt_axis(RadixList<Rs...>, cx<T> *tile, const cx<T> *tw) {
+  zt_stages<T, NZ, NTT, ALONG_T, INV, ALONG_T ? NTT : NZ, Rs...>(tile, tw);
+}
+
+template <typename T, int NZ, int NTT>
+__global__ void __launch_bounds__(ZtTile<NZ, NTT>::threads) k_fx_zt(T *__restrict__ data, int64_t V, int64_t nxy,
+                                                                   FFTTables tb, const Ctrl *ctrl, int check_active,
+                                                                   int tkid) {
+  static_assert(std::is_same<T, float>::value, "float pass");
+  follow_on();
+  data += (int64_t)blockIdx.z * 4 * V * 2;
+  ctrl += blockIdx.z;
+  if (!should_run<T>(ctrl, check_active)) return;
+  count_run(ctrl, tkid);
+  using Z = ZtTile<NZ, NTT>;
+  constexpr int C = Z::C, NTHR = Z::threads, CHUNKS = Z::NEL / 2, PER_ROW = C / 2;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cx<T> *tile = reinterpret_cast<cx<T> *>(smem_raw);
+  cx<T> *twz = tile + NTT * Z::PZ * C, *twt = twz + NZ;
+  T *sxyz = reinterpret_cast<T *>(twt + NTT), *srow = sxyz + NZ * C;
+  const int64_t col0 = (int64_t)blockIdx.x * C;
+  float2 *fld = reinterpret_cast<float2 *>(data + (int64_t)blockIdx.y * V * 2) + col0;
+  for (int i = threadIdx.x; i < CHUNKS; i += NTHR) {
+    const int row = i / PER_ROW, q = 2 * (i % PER_ROW);
+    cp_async16(tile + Z::at(row / NZ, row % NZ) + q, fld + row * nxy + q);
+  }
+  cp_async_commit();
+  load_twiddles<T, NZ>(twz, tb.tw[2]);
+  load_twiddles<T, NTT>(twt, tb.tw[3]);
+  // weight of each (t, z, column): w = p2max / (V (p2_xyz + p2_t)), 0 at k = 0
+  for (int i = threadIdx.x; i < NZ * C; i += NTHR) {
+    const unsigned q = (unsigned)col0 + i % C, x = q % (unsigned)tb.n[0], y = q / (unsigned)tb.n[0];
+    sxyz[i] = convert<T>(__ldg(tb.p2part[0] + x) + __ldg(tb.p2part[1] + y) + __ldg(tb.p2part[2] + i / C));
+  }
+  for (int i = threadIdx.x; i < NTT; i += NTHR) srow[i] = convert<T>(__ldg(tb.p2part[3] + i));
+  cp_async_wait_all();
+  __syncthreads();
+  using PlanZ = typename PlanOf<NZ>::type;
+  using PlanT = typename PlanOf<NTT>::type;
+  zt_axis<T, NZ, NTT, false, false>(PlanZ{}, tile, twz);
+  zt_axis<T, NZ, NTT, true, false>(PlanT{}, tile, twt);
+  {
+    const T wscale = convert<T>(tb.wscale);
+    const T zero = kconst<T>(0.0);
+#pragma unroll 4
+    for (int e = threadIdx.x; e < Z::NEL; e += NTHR) {
+      const int zc = e % (NZ * C), t = e / (NZ * C);
+      const T p2 = sxyz[zc] + srow[t];
+      const T w = p2 == zero ? zero : wscale / p2;
+      cx<T> &v = tile[Z::at(t, zc / C) + zc % C];
+      v = scale(v, w);
+    }
+    __syncthreads();
+  }
+  zt_axis<T, NZ, NTT, true, true>(PlanT{}, tile, twt);
+  zt_axis<T, NZ, NTT, false, true>(PlanZ{}, tile, twz);
+  for (int i = threadIdx.x; i < CHUNKS; i += NTHR) {
+    const int row = i / PER_ROW, q = 2 * (i % PER_ROW);
+    *reinterpret_cast<float4 *>(fld + row * nxy + q) =
+        *reinterpret_cast<const float4 *>(tile + Z::at(row / NZ, row % NZ) + q);
+  }
+}
+
 }  // namespace lgf

@@ -82,6 +82,7 @@ struct Pass {
   int kind = 0;
   int N = 0, C = 0, mode = 0, twmu = 0, ncb = 0, nblocks = 0;
   int64_t rstride = 0, ostride = 0;
+  const void *kernel = nullptr;  // kind 5: z and t with the filter (k_fx_zt)
   int grid_x = 0;  // blocks launched along x: one wave of the GPU (each block loops over its tiles), or nblocks
 };
 constexpr int kFixedThreads = 256;
@@ -154,6 +155,7 @@ struct lgf_ctx {
   int num_sms = 1;
   bool fft_persist = true;   // specialised FFT passes as one wave of tile-looping blocks (LGF_FFT_PERSIST=0: off)
   bool tfilter_reg = true;   // float t pass with the filter in registers at Nt = 64 (LGF_TFILTER_REG=0: off)
+  bool fft_zt = true;        // float z and t passes with the filter as one (LGF_FFT_ZT=0: off)
   bool xy_reg = true;        // float 64 x 64 xy passes in registers (LGF_XY_REG=0: off)
   bool twalk = true;  // float and residual Delta and updates walking along t (LGF_TWALK=0: off; twalk_on)
   int64_t twalk_min_blocks = 2048;  // LGF_TWALK_MIN_BLOCKS
@@ -320,7 +322,9 @@ template <typename T> lgf_status alloc(lgf_ctx *ctx, T **p, size_t count) {
 }
 
 // Kernel pointers of the specialised passes (instantiated in the per-type FFT translation units).
-template <typename T> const void *fixed_kernel(const Pass &p) { return fft_fixed_kernel<T>(p.kind, p.mode, p.N, p.C); }
+template <typename T> const void *fixed_kernel(const Pass &p) {
+  return p.kernel ? p.kernel : fft_fixed_kernel<T>(p.kind, p.mode, p.N, p.C);
+}
 
 // Specialised plan (5 passes: xy forward, z forward, t forward + filter + inverse, z inverse,
 // xy inverse) when every extent is one of the fixed lengths and Nx == Ny; false otherwise.
@@ -375,6 +379,22 @@ template <typename T> bool plan_fixed(lgf_ctx *ctx, State<T> &S) {
   }
   S.passes.clear();
   S.passes.push_back(plane(0, KID_FFT_XY_FWD));
+  if (sizeof(T) == 4 && ctx->fft_zt && Nz * Nt <= kZtSites) {  // one pass for z, t and the filter
+    const ZtKernel k = fft_float_zt(Nz, Nt);
+    Pass p{};
+    p.kind = 5;
+    p.kernel = k.kernel;
+    p.mode = 2;
+    p.C = k.C;
+    p.kid = KID_FFT_ZT_FILTER;
+    p.rstride = Nxy;
+    p.nblocks = (int)(Nxy / k.C);
+    p.threads = k.threads;
+    p.smem = k.smem;
+    S.passes.push_back(p);
+    S.passes.push_back(plane(1, KID_FFT_XY_INV));
+    return true;
+  }
   S.passes.push_back(cols(Nz, 0, Nxy, (int)(Nxy / C), Nxyz, Nt, 2, KID_FFT_Z_FWD));
   S.passes.push_back(cols(Nt, 2, Nxyz, (int)(Nxyz / C), 0, 1, 3, KID_FFT_T_FILTER));
   if (sizeof(T) == 4 && Nt == 64 && C == 32 && ctx->tfilter_reg) {
@@ -552,7 +572,7 @@ template <typename T> lgf_status opt_in_smem(lgf_ctx *ctx, State<T> &S) {
                                              : p.mode == 1 ? prefetch_tiles<FT, 2, 1>()
                                                            : prefetch_tiles<FT, 2, 2>())
                                           : prefetch_tiles<FT, 1, 0>();  // kind 1 and 3: one tile per block
-        p.grid_x = ctx->fft_persist && prefetch ? (int)std::min<int64_t>(p.nblocks, std::max<int64_t>(gx, 1))
+        p.grid_x = p.kind != 5 && ctx->fft_persist && prefetch ? (int)std::min<int64_t>(p.nblocks, std::max<int64_t>(gx, 1))
                                                 : p.nblocks;
       }
     }
@@ -782,6 +802,12 @@ template <typename T> lgf_status launch_filter(lgf_ctx *ctx, State<T> &S, T *dat
       const Ctrl *c = ctx->ctrl;
       void *args[] = {&data, &V, &pd, &tb, &c, &check_active, (void *)&tk};
       TRY(launch_next_ptr(ctx, fft_generic_kernel<FT>(), grid, p.threads, p.smem, args));
+    } else if (p.kind == 5) {
+      int64_t V = ctx->V, nxy = p.rstride;
+      FFTTables tb = S.tables;
+      const Ctrl *c = ctx->ctrl;
+      void *args[] = {&data, &V, &nxy, &tb, &c, &check_active, (void *)&tk};
+      TRY(launch_next_ptr(ctx, fixed_kernel<FT>(p), dim3(p.nblocks, 4, ctx->nb), p.threads, p.smem, args));
     } else if (p.kind == 1 || p.kind == 4) {
       dim3 grid(p.grid_x > 0 ? p.grid_x : p.nblocks, 4, ctx->nb);
       int64_t V = ctx->V;
@@ -1252,6 +1278,8 @@ static lgf_status create_ctx(const int n[4], int nb, lgf_ctx **out) {
     ctx->fft_persist = !(fp && fp[0] == '0');
     const char *tr = std::getenv("LGF_TFILTER_REG");
     ctx->tfilter_reg = !(tr && tr[0] == '0');
+    const char *zt = std::getenv("LGF_FFT_ZT");
+    ctx->fft_zt = !(zt && zt[0] == '0');
     const char *xr = std::getenv("LGF_XY_REG");
     ctx->xy_reg = !(xr && xr[0] == '0');
     const char *tw = std::getenv("LGF_TWALK");
