@@ -623,12 +623,18 @@ __global__ void __launch_bounds__(NT) k_gauge(const PT *__restrict__ P, T *__res
   }
 }
 
-// A = g - 1 in double-float from a g field (the single-step update takes g from the caller).
-template <int NT> __global__ void k_a_from_g(const double *__restrict__ G, float *__restrict__ A, int64_t V) {
+// The caller's g (matrices) in planes, and A = g - 1 in double-float, for the single-step update.
+template <int NT>
+__global__ void __launch_bounds__(NT) k_g_planes(const double *__restrict__ g, double *__restrict__ G,
+                                                float *__restrict__ A, int64_t V) {
   const int64_t s = (int64_t)blockIdx.x * NT + threadIdx.x;
   if (s >= V) return;
 #pragma unroll
-  for (int e = 0; e < 9; ++e) st_a(A, (int64_t)e * V + s, minus_identity_split(ldg(G, (int64_t)e * V + s), e));
+  for (int e = 0; e < 9; ++e) {
+    const cx<double> v = ldg(g, s * 9 + e);
+    st(G, (int64_t)e * V + s, v);
+    st_a(A, (int64_t)e * V + s, minus_identity_split(v, e));
+  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -669,11 +675,15 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // so that four blocks of 128 threads (16 warps) fit on an SM.
 template <int NT> constexpr size_t update_smem_bytes() { return (size_t)27 * NT * 16; }
 
-template <int NT>
+// Element e of the link of site s of one direction: planes, or (AOS) the caller's matrices.
+template <bool AOS> __device__ __forceinline__ int64_t link_at(int e, int64_t V, int64_t s) {
+  return AOS ? s * 9 + e : (int64_t)e * V + s;
+}
+template <int NT, bool AOS>
 __device__ __forceinline__ void fetch_u(const double *plane, int64_t V, int64_t s, double2 *bu) {
   const double2 *pu = reinterpret_cast<const double2 *>(plane);
 #pragma unroll
-  for (int e = 0; e < 9; ++e) cp_async16(bu + e * NT + threadIdx.x, pu + (int64_t)e * V + s);
+  for (int e = 0; e < 9; ++e) cp_async16(bu + e * NT + threadIdx.x, pu + link_at<AOS>(e, V, s));
   cp_async_commit();
 }
 template <int NT>
@@ -684,14 +694,14 @@ __device__ __forceinline__ void fetch_b(const float *A, int64_t V, int64_t sf, f
   cp_async_commit();
 }
 // Start the copies of link mu at site s (9 elements to bu) and of b at its forward neighbour sf (to bb).
-template <int NT>
+template <int NT, bool AOS>
 __device__ __forceinline__ void fetch_link(const double *plane, const float *A, int64_t V, int64_t s, int64_t sf,
                                            double2 *bu, float4 *bb) {
   const double2 *pu = reinterpret_cast<const double2 *>(plane);
   const float4 *pa = reinterpret_cast<const float4 *>(A);
 #pragma unroll
   for (int e = 0; e < 9; ++e) {
-    cp_async16(bu + e * NT + threadIdx.x, pu + (int64_t)e * V + s);
+    cp_async16(bu + e * NT + threadIdx.x, pu + link_at<AOS>(e, V, s));
     cp_async16(bb + e * NT + threadIdx.x, pa + (int64_t)e * V + sf);
   }
   cp_async_commit();
@@ -699,7 +709,7 @@ __device__ __forceinline__ void fetch_link(const double *plane, const float *A, 
 
 // Small-step update of one link: u (the link) and b = g(x+mu) - 1 in double-float registers, a (rows of
 // g(x) - 1) in shared memory, the FP64 link in bu; the new link is stored to the plane.
-template <int NT>
+template <int NT, bool AOS>
 __device__ __forceinline__ void update_link_small(double *plane, int64_t V, int64_t s, const float4 *sa,
                                                   double2 *bu, const cx<df64> u[9], const cx<df64> b[9]) {
   // rows 0 and 1 one at a time (a rolled loop keeps the code within the instruction cache); each new
@@ -742,7 +752,7 @@ __device__ __forceinline__ void update_link_small(double *plane, int64_t V, int6
       const double2 old = bu[e * NT + threadIdx.x];
       const double2 nu = make_double2(old.x + df64_widen(dfacc_result(re)), old.y + df64_widen(dfacc_result(im)));
       bu[e * NT + threadIdx.x] = nu;
-      st(plane, (int64_t)e * V + s, from_vec<double>(nu));
+      st(plane, link_at<AOS>(e, V, s), from_vec<double>(nu));
     }
   }
   // row 2 = conj(row0 x row1) in FP64, as in the general form (the FP64 pipe has room here)
@@ -752,9 +762,9 @@ __device__ __forceinline__ void update_link_small(double *plane, int64_t V, int6
     r0[j] = from_vec<double>(bu[j * NT + threadIdx.x]);
     r1[j] = from_vec<double>(bu[(3 + j) * NT + threadIdx.x]);
   }
-  st(plane, 6 * V + s, cross_cj(r0[1], r1[2], r0[2], r1[1]));
-  st(plane, 7 * V + s, cross_cj(r0[2], r1[0], r0[0], r1[2]));
-  st(plane, 8 * V + s, cross_cj(r0[0], r1[1], r0[1], r1[0]));
+  st(plane, link_at<AOS>(6, V, s), cross_cj(r0[1], r1[2], r0[2], r1[1]));
+  st(plane, link_at<AOS>(7, V, s), cross_cj(r0[2], r1[0], r0[0], r1[2]));
+  st(plane, link_at<AOS>(8, V, s), cross_cj(r0[0], r1[1], r0[1], r1[0]));
 }
 
 // General-step update of the links mu0 .. 3 of a site: rows 0 and 1 of g(x) U g^+(x+mu) in 60-bit fixed
@@ -763,7 +773,7 @@ __device__ __forceinline__ void update_link_small(double *plane, int64_t V, int6
 // per thread: the loops over columns are rolled and keep the limbs of g(x) U (in oth) and of the result (in
 // cur) in shared memory, because the unrolled form, 3000 instructions a link, waited for its own code. While
 // row 2 is formed the next link and g are copied to oth and gs.
-template <int NT>
+template <int NT, bool AOS>
 __device__ __forceinline__ void update_links_general(double *U, const double *G, const Lattice &L, int64_t s,
                                                      const int c[4], int mu0, int nf, int4 *cur, int4 *oth,
                                                      int4 *gs) {
@@ -771,14 +781,16 @@ __device__ __forceinline__ void update_links_general(double *U, const double *G,
   cur += threadIdx.x;
   oth += threadIdx.x;
   gs += threadIdx.x;
-  auto fetch = [&](const double *src, int64_t at, int4 *dst) {
-    const int4 *p = reinterpret_cast<const int4 *>(src) + at;
+  auto fetch = [&](auto aos, const double *src, int64_t at, int4 *dst) {
+    const int4 *p = reinterpret_cast<const int4 *>(src);
 #pragma unroll
-    for (int e = 0; e < 9; ++e) cp_async16(dst + e * NT, p + (int64_t)e * V);
+    for (int e = 0; e < 9; ++e) cp_async16(dst + e * NT, p + link_at<aos.value>(e, V, at));
     cp_async_commit();
   };
+  constexpr std::false_type planes{};
+  constexpr std::integral_constant<bool, AOS> links{};
   const int4 *gp = reinterpret_cast<const int4 *>(G) + s;
-  fetch(G, site_fwd(L, s, mu0, c[mu0]), gs);
+  fetch(planes, G, site_fwd(L, s, mu0, c[mu0]), gs);
   clq gx[6];
   int topx = 0;
 #pragma unroll
@@ -790,11 +802,11 @@ __device__ __forceinline__ void update_links_general(double *U, const double *G,
 #pragma unroll 1
   for (int mu = mu0; mu < 4; ++mu) {
     double *plane = U + (int64_t)mu * pstride;
-    auto out = [&](int e, cx<double> v) { st(plane, (int64_t)e * V + s, v); };
+    auto out = [&](int e, cx<double> v) { st(plane, link_at<AOS>(e, V, s), v); };
     auto next = [&]() {
       if (mu == 3) return;
-      fetch(plane + pstride, s, oth);
-      fetch(G, site_fwd(L, s, mu + 1, c[mu + 1]), gs);
+      fetch(links, plane + pstride, s, oth);
+      fetch(planes, G, site_fwd(L, s, mu + 1, c[mu + 1]), gs);
     };
     cp_async_wait_all();
     int top = topx;
@@ -861,7 +873,7 @@ __device__ __forceinline__ void update_links_general(double *U, const double *G,
 // one direction in every other warp in FP64, 0.49 with two in every warp and 0.57 with two in the 61-bit form
 // of q61.cuh, which joins and splits the limbs at every product. The integer and conversion instructions
 // bound it (16 warps per SM, the bytes would take 0.13 ms).
-template <typename T, int NT>
+template <typename T, int NT, bool AOS = false>
 __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 4 : 2)
     k_update(T *__restrict__ U, const T *__restrict__ G, const float *__restrict__ A, Lattice L, const Ctrl *ctrl,
              int check_active, int tkid, int allow_small, int fp64_even, int fp64_odd) {
@@ -893,7 +905,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 4 : 2)
 #pragma unroll
       for (int e = 0; e < 9; ++e) cp_async16(sa + e * NT + threadIdx.x, pa + (int64_t)e * V + s);
     }
-    fetch_link<NT>(U, A, V, s, site_fwd(L, s, 0, c[0]), bu0, bb);
+    fetch_link<NT, AOS>(U, A, V, s, site_fwd(L, s, 0, c[0]), bu0, bb);
     cp_async_wait_all();
     int ea = 0;
 #pragma unroll
@@ -920,11 +932,11 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 4 : 2)
         u[e] = {df64_split_fast(v.x), df64_split_fast(v.y)};
       }
       if (mu < 3) fetch_b<NT>(A, V, site_fwd(L, s, mu + 1, c[mu + 1]), bb);
-      update_link_small<NT>(plane, V, s, sa, bu0, u, b);
-      if (mu < 3) fetch_u<NT>(plane + pstride, V, s, bu0);
+      update_link_small<NT, AOS>(plane, V, s, sa, bu0, u, b);
+      if (mu < 3) fetch_u<NT, AOS>(plane + pstride, V, s, bu0);
     }
     if (mu < 4)
-      update_links_general<NT>(U, G, L, s, c, mu, ((threadIdx.x >> 5) & 1) ? fp64_odd : fp64_even,
+      update_links_general<NT, AOS>(U, G, L, s, c, mu, ((threadIdx.x >> 5) & 1) ? fp64_odd : fp64_even,
                                reinterpret_cast<int4 *>(bu0), reinterpret_cast<int4 *>(sa),
                                reinterpret_cast<int4 *>(bb));
   } else {
