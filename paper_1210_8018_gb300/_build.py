@@ -6,7 +6,8 @@ import subprocess
 HERE = os.path.dirname(os.path.abspath(__file__))
 SO = os.path.join(HERE, "liblgf.so")
 SOURCES = [os.path.join(HERE, "csrc", f) for f in
-           ("lgf.cu", "noalloc.cu", "fft_float.cu", "fft_float_zt.cu", "fft_double.cu", "fft_df64_planes.cu", "fft_df64_columns.cu")]
+           ("lgf.cu", "noalloc.cu", "fft_float.cu", "fft_float_zt.cu", "fft_df64_zt.cu",
+            "fft_df64_zt_long.cu", "fft_double.cu", "fft_df64_planes.cu", "fft_df64_columns.cu")]
 DEPS = [os.path.join(HERE, "csrc", f) for f in os.listdir(os.path.join(HERE, "csrc"))] + [
     os.path.join(os.path.dirname(HERE), "include", "lgf.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo", "-std=c++17",

@@ -1,0 +1,13 @@
+// fft_df64_zt_long.cu -- the df64 passes over z and t for Nz above 16 (compiled apart).
+#include "fft_zt_instances.cuh"
+
+namespace lgf {
+ZtKernel fft_df64_zt_long(int nz, int nt) {
+  switch (nz) {
+    case 24: return zt_by_nt<df64, 24>(nt);
+    case 32: return zt_by_nt<df64, 32>(nt);
+    case 48: return zt_by_nt<df64, 48>(nt);
+    default: return zt_by_nt<df64, 64>(nt);
+  }
+}
+}  // namespace lgf

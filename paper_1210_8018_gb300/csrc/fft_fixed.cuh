@@ -538,24 +538,22 @@ __global__ void __launch_bounds__(NT, 5) k_fx_tfilter64(T *__restrict__ data, in
 // k_fx_cols, and what it rounds when it stores a field is rounded here in the tile: the same bits.
 // Tile: element (t, z, c) at (t PZ + z + z / 8) C + c. Threads run through c, then j or the block of a z stage
 // (the padding after every eighth z keeps the last stage, which strides by its radix, free of bank conflicts), then
-// t; in the t stages through c, z, then the rest. The trips through shared memory bound it, which is why the
-// planner takes it up to Nz Nt = kZtSites only. Measured per iteration, with the events of the timing mode, against
-// the three column passes: 16 x 32 (16^3 x 32) 16 against 35 us, 32 x 32 (32^4) 44 / 68, 32 x 48 (48^2 x 32 x 48)
-// 155 / 181, 32 x 64 (64^2 x 32 x 64) 289 / 323; but 48 x 48 (48^4) 299 / 277, 64 x 64 (64^4) 621 / 572.
-// Mixed fix at 8^4 1.28 -> 1.15 ms, 16^3 x 32 2.82 -> 2.65, 32^4 14.0 -> 13.7.
+// t; in the t stages through c, z, then the rest. The trips through shared memory bound it, in df64 the
+// arithmetic: zt_faster says where it is planned. Mixed fix at 8^4 1.28 -> 1.15 ms, 16^3 x 32 2.82 -> 2.65,
+// 32^4 14.0 -> 13.6; ensemble of six 16^4 in double 23.7 -> 22.8.
 // ---------------------------------------------------------------------------------------------
-template <int NZ, int NTT> struct ZtTile {
-  // 64-byte runs in the small tiles, else 32-byte runs (32 x 32: 44 us against 48 with 64-byte runs at 32^4)
-  static constexpr int C = NZ * NTT <= 768 ? 8 : 4;
+template <typename T, int NZ, int NTT> struct ZtTile {
+  // 64-byte runs in the small tiles, else 32-byte runs (float 32 x 32: 44 us against 48 with 64-byte runs at 32^4)
+  static constexpr int C = (NZ * NTT <= 768 ? 64 : 32) / (int)sizeof(cx<T>);
   static constexpr int PZ = NZ + NZ / 8;
   static constexpr int NEL = NZ * NTT * C;
   static constexpr int threads = NEL >= 6144 ? 512 : 256;
-  static constexpr size_t smem = (size_t)(NTT * PZ * C + NZ + NTT) * 8 + (size_t)(NZ * C + NTT) * 4;
+  static constexpr size_t smem = (size_t)(NTT * PZ * C + NZ + NTT) * sizeof(cx<T>) + (size_t)(NZ * C + NTT) * sizeof(T);
   __device__ static __forceinline__ int at(int t, int z) { return (t * PZ + z + (z >> 3)) * C; }
 };
 template <typename T, int NZ, int NTT, bool ALONG_T, int L, int R, bool INV>
 __device__ __forceinline__ void zt_stage(cx<T> *tile, const cx<T> *tw) {
-  using Z = ZtTile<NZ, NTT>;
+  using Z = ZtTile<T, NZ, NTT>;
   constexpr int C = Z::C, N = ALONG_T ? NTT : NZ, M = L / R, NB = N / R, TWSTEP = N / L, ITEMS = Z::NEL / R;
 #pragma unroll 2
   for (int w = threadIdx.x; w < ITEMS; w += Z::threads) {
@@ -599,25 +597,25 @@ __device__ __forceinline__ void zt_axis(RadixList<Rs...>, cx<T> *tile, const cx<
 }
 
 template <typename T, int NZ, int NTT>
-__global__ void __launch_bounds__(ZtTile<NZ, NTT>::threads) k_fx_zt(T *__restrict__ data, int64_t V, int64_t nxy,
+__global__ void __launch_bounds__(ZtTile<T, NZ, NTT>::threads) k_fx_zt(T *__restrict__ data, int64_t V, int64_t nxy,
                                                                    FFTTables tb, const Ctrl *ctrl, int check_active,
                                                                    int tkid) {
-  static_assert(std::is_same<T, float>::value, "float pass");
   follow_on();
   data += (int64_t)blockIdx.z * 4 * V * 2;
   ctrl += blockIdx.z;
   if (!should_run<T>(ctrl, check_active)) return;
   count_run(ctrl, tkid);
-  using Z = ZtTile<NZ, NTT>;
-  constexpr int C = Z::C, NTHR = Z::threads, CHUNKS = Z::NEL / 2, PER_ROW = C / 2;
+  using Z = ZtTile<T, NZ, NTT>;
+  constexpr int C = Z::C, NTHR = Z::threads;
+  constexpr int W = 16 / (int)sizeof(cx<T>), CHUNKS = Z::NEL / W, PER_ROW = C / W;  // elements per 16 bytes
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T> *tile = reinterpret_cast<cx<T> *>(smem_raw);
   cx<T> *twz = tile + NTT * Z::PZ * C, *twt = twz + NZ;
   T *sxyz = reinterpret_cast<T *>(twt + NTT), *srow = sxyz + NZ * C;
   const int64_t col0 = (int64_t)blockIdx.x * C;
-  float2 *fld = reinterpret_cast<float2 *>(data + (int64_t)blockIdx.y * V * 2) + col0;
+  cx<T> *fld = reinterpret_cast<cx<T> *>(data + (int64_t)blockIdx.y * V * 2) + col0;
   for (int i = threadIdx.x; i < CHUNKS; i += NTHR) {
-    const int row = i / PER_ROW, q = 2 * (i % PER_ROW);
+    const int row = i / PER_ROW, q = W * (i % PER_ROW);
     cp_async16(tile + Z::at(row / NZ, row % NZ) + q, fld + row * nxy + q);
   }
   cp_async_commit();
@@ -651,7 +649,7 @@ __global__ void __launch_bounds__(ZtTile<NZ, NTT>::threads) k_fx_zt(T *__restric
   zt_axis<T, NZ, NTT, true, true>(PlanT{}, tile, twt);
   zt_axis<T, NZ, NTT, false, true>(PlanZ{}, tile, twz);
   for (int i = threadIdx.x; i < CHUNKS; i += NTHR) {
-    const int row = i / PER_ROW, q = 2 * (i % PER_ROW);
+    const int row = i / PER_ROW, q = W * (i % PER_ROW);
     *reinterpret_cast<float4 *>(fld + row * nxy + q) =
         *reinterpret_cast<const float4 *>(tile + Z::at(row / NZ, row % NZ) + q);
   }

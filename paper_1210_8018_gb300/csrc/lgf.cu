@@ -156,7 +156,7 @@ struct lgf_ctx {
   int num_sms = 1;
   bool fft_persist = true;   // specialised FFT passes as one wave of tile-looping blocks (LGF_FFT_PERSIST=0: off)
   bool tfilter_reg = true;   // float t pass with the filter in registers at Nt = 64 (LGF_TFILTER_REG=0: off)
-  bool fft_zt = true;        // float z and t passes with the filter as one (LGF_FFT_ZT=0: off)
+  bool fft_zt = true;        // z and t passes with the filter as one (LGF_FFT_ZT=0: off)
   bool xy_reg = true;        // float 64 x 64 xy passes in registers (LGF_XY_REG=0: off)
   bool twalk = true;  // float and residual Delta and updates walking along t (LGF_TWALK=0: off; twalk_on)
   int64_t twalk_min_blocks = 2048;  // LGF_TWALK_MIN_BLOCKS
@@ -380,8 +380,11 @@ template <typename T> bool plan_fixed(lgf_ctx *ctx, State<T> &S) {
   }
   S.passes.clear();
   S.passes.push_back(plane(0, KID_FFT_XY_FWD));
-  if (sizeof(T) == 4 && ctx->fft_zt && Nz * Nt <= kZtSites) {  // one pass for z, t and the filter
-    const ZtKernel k = fft_float_zt(Nz, Nt);
+  // one pass for z, t and the filter where there is a kernel for it
+  ZtKernel k{};
+  if (ctx->fft_zt && sizeof(T) == 4) k = fft_float_zt(Nz, Nt);
+  else if (ctx->fft_zt && ctx->fft_df64) k = fft_df64_zt(Nz, Nt);
+  if (k.kernel && Nxy % k.C == 0) {
     Pass p{};
     p.kind = 5;
     p.kernel = k.kernel;

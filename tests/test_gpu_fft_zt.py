@@ -1,4 +1,4 @@
-"""The float pass over z and t with the filter (k_fx_zt) against the three column passes (LGF_FFT_ZT=0): the same
+"""The pass over z and t with the filter (k_fx_zt), in float and double-float, against the three column passes (LGF_FFT_ZT=0): the same
 bits for every pair of extents that takes it and for the pairs beside its limit, and for a batch."""
 import numpy as np
 import pytest
@@ -8,8 +8,9 @@ pytestmark = pytest.mark.gpu
 PAIRS = [(nz, nt) for nz in (8, 16, 24, 32, 48, 64) for nt in (8, 16, 24, 32, 48, 64)]
 
 
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
 @pytest.mark.parametrize("nxy", [8, 24])
-def test_same_bits_as_column_passes(nxy, monkeypatch):
+def test_same_bits_as_column_passes(nxy, precision, monkeypatch):
     import torch
 
     import paper_1210_8018_gb300 as lgf
@@ -23,7 +24,7 @@ def test_same_bits_as_column_passes(nxy, monkeypatch):
             monkeypatch.setenv("LGF_FFT_ZT", flag)
             with lgf.Lattice((nxy, nxy, nz, nt)) as lat:
                 out.append(torch.empty_like(d))
-                lat.filter(d, out[-1], "fp32")
+                lat.filter(d, out[-1], precision)
         assert torch.equal(out[0], out[1]), (nz, nt)
 
 
