@@ -172,13 +172,14 @@ lgf_status lgf_filter_coeffs(lgf_ctx *ctx, const double *coef, double *out, int 
 /* ---- The functional as a differentiable function of a Lie-algebra field (Eq. 1 at g = exp(i omega)).
  * omega: V*8 doubles, site-major: omega[8*s + a] is the coefficient of T^a = lambda^a/2 (Gell-Mann
  * matrices), so omega(x) = sum_a omega^a T^a is Hermitian and traceless; g(x) = exp(i omega(x)) is
- * formed from a Jacobi eigen-decomposition of omega(x). Pointers may be device or host pointers. ---- */
+ * formed by its series (from a Jacobi eigen-decomposition of omega(x) above a Frobenius norm of 64). Pointers may
+ * be device or host pointers. ---- */
 
 /* F = F_U[exp(i omega)] (Eq. 1); g_out (V*9 complex, site-field layout) receives g if not NULL. */
 lgf_status lgf_functional(lgf_ctx *ctx, const double *links, const double *omega, double *F, double *g_out);
 
 /* grad[8*s + a] = scale * dF/d omega^a(s): the su(3) gradient, i.e. the steepest-ascent direction
- * (Daleckii-Krein adjoint of the exponential applied to the staple of Eq. 1). At omega = 0 it equals
+ * (the adjoint of the exponential's derivative applied to the staple of Eq. 1). At omega = 0 it equals
  * -scale * (i / (24 V)) Tr[T^a Delta(s)] with Delta of Eq. 5. */
 lgf_status lgf_functional_grad(lgf_ctx *ctx, const double *links, const double *omega, double scale, double *grad);
 
