@@ -172,7 +172,7 @@ lgf_status lgf_filter_coeffs(lgf_ctx *ctx, const double *coef, double *out, int 
 /* ---- The functional as a differentiable function of a Lie-algebra field (Eq. 1 at g = exp(i omega)).
  * omega: V*8 doubles, site-major: omega[8*s + a] is the coefficient of T^a = lambda^a/2 (Gell-Mann
  * matrices), so omega(x) = sum_a omega^a T^a is Hermitian and traceless; g(x) = exp(i omega(x)) is
- * formed by its series (from a Jacobi eigen-decomposition of omega(x) above a Frobenius norm of 64). Pointers may
+ * formed by its series (from a Jacobi eigen-decomposition of omega(x) above a Frobenius norm of 3). Pointers may
  * be device or host pointers. ---- */
 
 /* F = F_U[exp(i omega)] (Eq. 1); g_out (V*9 complex, site-field layout) receives g if not NULL. */

@@ -36,7 +36,7 @@ def reference(U, w):
     return float(F), grad.numpy().reshape(-1, 8)
 
 
-# norms of omega are 2 * size: no doubling, one to eight doublings, eigenvectors
+# norms of omega are 2 * size: no doubling, doublings, eigenvectors
 @pytest.mark.parametrize("size", [0.0, 1e-9, 0.02, 0.2, 0.26, 1.0, 7.0, 31.0, 33.0, 60.0])
 @pytest.mark.parametrize("links", ["su3", "scaled"])
 def test_functional_and_gradient(size, links):
