@@ -14,6 +14,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <type_traits>
 #include <vector>
@@ -554,18 +555,27 @@ template <> void fill_twiddles<df64>(std::vector<df64> &tw, int N) {
   }
 }
 
-// Opt the FFT kernels in to the dynamic shared memory each pass needs (the generic kernel: the
-// largest of its passes).
+// Opt a kernel in to `bytes` of dynamic shared memory. The limit belongs to the kernel, not to the context, and
+// other contexts (or the other groups of a batch) have plans of their own for it: it only ever rises.
+lgf_status raise_smem_limit(lgf_ctx *ctx, const void *kernel, size_t bytes) {
+  static std::mutex mutex;  // between the look and the rise
+  if (bytes <= 48 * 1024) return LGF_OK;
+  std::lock_guard<std::mutex> lock(mutex);
+  cudaFuncAttributes a;
+  CK(cudaFuncGetAttributes(&a, kernel));
+  if ((size_t)a.maxDynamicSharedSizeBytes < bytes)
+    CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  return LGF_OK;
+}
+
+// Opt the FFT kernels in to the dynamic shared memory each pass needs.
 // The specialised passes get one wave of blocks (resident blocks per SM x SMs, over the fields and the
 // configurations of the launch), each looping over its tiles with the next tile's loads in flight.
 template <typename T> lgf_status opt_in_smem(lgf_ctx *ctx, State<T> &S) {
   return with_fft_type<T>(ctx, [&](auto tag) -> lgf_status {
     using FT = decltype(tag);
-    size_t generic_max = 0;
     for (auto &p : S.passes) {
-      if (p.kind == 0) generic_max = std::max(generic_max, p.smem);
-      else if (p.smem > 48 * 1024)
-        CK(cudaFuncSetAttribute(fixed_kernel<FT>(p), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem));
+      TRY(raise_smem_limit(ctx, p.kind == 0 ? fft_generic_kernel<FT>() : fixed_kernel<FT>(p), p.smem));
       if (p.kind != 0) {
         int per_sm = 0;
         CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fixed_kernel<FT>(p), p.threads, p.smem));
@@ -580,8 +590,6 @@ template <typename T> lgf_status opt_in_smem(lgf_ctx *ctx, State<T> &S) {
                                                 : p.nblocks;
       }
     }
-    if (generic_max > 48 * 1024)
-      CK(cudaFuncSetAttribute(fft_generic_kernel<FT>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)generic_max));
     return LGF_OK;
   });
 }
