@@ -13,7 +13,8 @@ namespace lgf {
 //
 // Range: with rows a and columns b of unit length (six real entries, sum |a_k| <= 6^(1/2)) the cross sum
 // stays below 2 * 2.45 * 2^60 < 2^63, and that holds up to sum |a_k| + sum |b_k| = 8. Callers send entries
-// of magnitude 2 and above, infinities and NaN (lq_in_range) to the FP64 form.
+// of magnitude 2 and above, infinities and NaN (lq_in_range), and matrices whose rows or columns are longer, to
+// the FP64 form.
 // Error: the dropped products of the low limbs are below 2^-60 each and the splits truncate by less than
 // 2^-60, so an element is off by less than 2^-57 before its one rounding to double.
 struct lq {
@@ -46,6 +47,10 @@ __device__ __forceinline__ void lmac(lacc &s, lq a, lq b) {
   s.c += (long long)a.l * b.h;
 }
 __device__ __forceinline__ long long lacc_value(lacc s) { return s.hh + (s.c >> 30); }  // times 2^-60
+// of two sums whose cross sums may not fit in 64 bits together (their mean does)
+__device__ __forceinline__ long long lacc_value(lacc s, lacc w) {
+  return s.hh + w.hh + (((s.c & w.c) + ((s.c ^ w.c) >> 1)) >> 29);
+}
 __device__ __forceinline__ lq lq_split(long long v) { return {(int)(v >> 30), (int)((unsigned)v & 0x3FFFFFFFu)}; }
 __device__ __forceinline__ long long lq_join(lq a) { return ((long long)a.h << 30) + a.l; }
 // v 2^-60 rounded to nearest

@@ -768,11 +768,49 @@ __device__ __forceinline__ void update_link_small(double *plane, int64_t V, int6
 }
 
 // General-step update of the links mu0 .. 3 of a site: rows 0 and 1 of g(x) U g^+(x+mu) in 60-bit fixed
-// point (q60.cuh), row 2 = conj(row0 x row1); in FP64 for the directions below nf and where an entry of the
-// warp is out of the fixed-point range. `cur` holds the first link and is with `oth` and `gs` nine slots each
+// point (q60.cuh), row 2 = conj(row0 x row1); in FP64 for the directions below nf and where a site of the
+// warp is not for the fixed point. `cur` holds the first link and is with `oth` and `gs` nine slots each
 // per thread: the loops over columns are rolled and keep the limbs of g(x) U (in oth) and of the result (in
 // cur) in shared memory, because the unrolled form, 3000 instructions a link, waited for its own code. While
 // row 2 is formed the next link and g are copied to oth and gs.
+//
+// What is for the fixed point: entries of magnitude below 2, rows of g of about unit length and a Frobenius
+// norm of U of at most 3.05^(1/2) (limb_norm counts), whatever the angles between them. Then a row t of g(x) U
+// is at most 1.76 long, its elements and those of the result are below 1.78, and the cross sums of both products
+// stay below 6^(1/2) (1.76 + 1.01) = 6.8 of 8 (times 2^60). In row 2 they stay below 2 (1.76 + 1.76) = 7.1 for a
+// unitary g, which k_gauge's is; the caller's (AOS) is not checked for its angles, so there the two products'
+// cross sums, 5.1 each, are kept apart. And no less than FP64 would hold: no row of g or column of U shorter than
+// 1/4, not both U and g(x) with all elements beside the diagonal below 2^-5 together, because the fixed point
+// truncates them at 2^-60, where FP64 products of such matrices would err by 2^-53 of those elements.
+struct limb_norm {  // squares of the limbs to 12 bits: 2^24 is a length of 1
+  static constexpr unsigned one = 1u << 24, shortest = one / 16, row = 17028874, matrix = 51170508, offdiag = 1u << 14;
+  __device__ static __forceinline__ unsigned of(clq a) {
+    const int x = a.r.h >> 18, y = a.i.h >> 18;
+    return (unsigned)(x * x + y * y);
+  }
+};
+// Rows of a matrix (words of doubles below 2, thread's slots NT apart) of about unit length, in float: a double
+// between 2^-127 and 2 has the low seven bits of its exponent in common with the float (below, a row may seem
+// longer than it is and goes to FP64).
+template <int NT> __device__ __forceinline__ bool unit_rows(const int4 *m) {
+  auto sq = [](int hi, float n) {
+    const float x = __uint_as_float(((unsigned)hi & 0x07FFFFFFu) << 3);
+    return fmaf(x, x, n);
+  };
+  float lo = 4.f, hi = 0.f;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    float n = 0.f;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int4 v = m[(3 * i + j) * NT];
+      n = sq(v.w, sq(v.y, n));
+    }
+    lo = fminf(lo, n);
+    hi = fmaxf(hi, n);
+  }
+  return lo >= 1.f / 16 && hi <= 1.015f;
+}
 template <int NT, bool AOS>
 __device__ __forceinline__ void update_links_general(double *U, const double *G, const Lattice &L, int64_t s,
                                                      const int c[4], int mu0, int nf, int4 *cur, int4 *oth,
@@ -793,12 +831,17 @@ __device__ __forceinline__ void update_links_general(double *U, const double *G,
   fetch(planes, G, site_fwd(L, s, mu0, c[mu0]), gs);
   clq gx[6];
   int topx = 0;
+  unsigned nx[2] = {0, 0}, offx = 0;
 #pragma unroll
   for (int e = 0; e < 6; ++e) {
     const int4 v = ldv(gp + (int64_t)e * V);
     topx |= v.y | v.w;
     gx[e] = words_clq(v);
+    const unsigned n = limb_norm::of(gx[e]);
+    nx[e / 3] += n;
+    if (e % 3 != e / 3) offx += n;
   }
+  if (min(nx[0], nx[1]) < limb_norm::shortest || max(nx[0], nx[1]) > limb_norm::row) topx = -1;
 #pragma unroll 1
   for (int mu = mu0; mu < 4; ++mu) {
     double *plane = U + (int64_t)mu * pstride;
@@ -815,24 +858,39 @@ __device__ __forceinline__ void update_links_general(double *U, const double *G,
       top |= cur[e * NT].y | cur[e * NT].w;
       top |= gs[e * NT].y | gs[e * NT].w;
     }
-    if (__any_sync(__activemask(), mu < nf || (top & 0x40000000))) {  // bit 30: a magnitude of 2 or more
+    bool fp64 = mu < nf || (top & 0x40000000);  // bit 30: a magnitude of 2 or more
+    if constexpr (AOS) fp64 |= !unit_rows<NT>(gs);
+    const unsigned warp = __activemask();
+    fp64 = __any_sync(warp, fp64);
+    if (!fp64) {
+      unsigned all = 0, least = ~0u, diag = 0;
+#pragma unroll 1
+      for (int j = 0; j < 3; ++j) {  // column j of rows 0-1 of g(x) U
+        clacc t[2] = {};
+        unsigned col = 0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const clq u = words_clq(cur[(3 * k + j) * NT]);
+          const unsigned n = limb_norm::of(u);
+          col += n;
+          diag += k == j ? n : 0;
+#pragma unroll
+          for (int i = 0; i < 2; ++i) clmac(t[i], gx[3 * i + k], u);
+        }
+        all += col;
+        least = min(least, col);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) oth[(3 * i + j) * NT] = to_int4(clacc_split(t[i]));
+      }
+      fp64 = __any_sync(warp, all > limb_norm::matrix || least < limb_norm::shortest ||
+                                  max(all - diag, offx) < limb_norm::offdiag);
+    }
+    if (fp64) {
       link_product_fp64([&](int e) { return words_double(ldv(gp + (int64_t)e * V)); },
                         [&](int e) { return words_double(cur[e * NT]); },
                         [&](int e) { return words_double(gs[e * NT]); }, out);
       next();
     } else {
-#pragma unroll 1
-      for (int j = 0; j < 3; ++j) {  // column j of rows 0-1 of g(x) U
-        clacc t[2] = {};
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const clq u = words_clq(cur[(3 * k + j) * NT]);
-#pragma unroll
-          for (int i = 0; i < 2; ++i) clmac(t[i], gx[3 * i + k], u);
-        }
-#pragma unroll
-        for (int i = 0; i < 2; ++i) oth[(3 * i + j) * NT] = to_int4(clacc_split(t[i]));
-      }
 #pragma unroll 1
       for (int j = 0; j < 3; ++j) {  // column j of rows 0-1 of the result, from row j of g(x + mu)
         clacc t[2] = {};
@@ -855,10 +913,17 @@ __device__ __forceinline__ void update_links_general(double *U, const double *G,
         const int j1 = j == 2 ? 0 : j + 1, j2 = j == 0 ? 2 : j - 1;
         const clq a = limbs_of(cur[j1 * NT]), b = limbs_of(cur[(3 + j2) * NT]);
         const clq d = limbs_of(cur[j2 * NT]), e = limbs_of(cur[(3 + j1) * NT]);
+        const clq ne = {lq_neg(e.r), lq_neg(e.i)};
         clacc t = {};  // a b - d e
         clmac(t, a, b);
-        clmac(t, d, {lq_neg(e.r), lq_neg(e.i)});
-        out(6 + j, {q60_double(lacc_value(t.re)), q60_double(-lacc_value(t.im))});
+        if constexpr (AOS) {
+          clacc w = {};
+          clmac(w, d, ne);
+          out(6 + j, {q60_double(lacc_value(t.re, w.re)), q60_double(-lacc_value(t.im, w.im))});
+        } else {
+          clmac(t, d, ne);
+          out(6 + j, {q60_double(lacc_value(t.re)), q60_double(-lacc_value(t.im))});
+        }
       }
     }
     int4 *const swap = cur;
