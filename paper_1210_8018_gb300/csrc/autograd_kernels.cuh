@@ -226,14 +226,14 @@ __device__ __noinline__ void expi_by_eigenvectors(const double *w, m3<double> *g
   expi_from_eig(W, l, *g);
 }
 
-// omega (V x 8, site-major) -> g in limb planes, and to the caller's g_out (array of structures) where asked.
+// omega (V x 8, site-major) -> g in limb planes, and where asked in planes of doubles.
 // A g that is not finite is marked by kNoLimb, which the readers turn into NaN.
 // Bound by the FP64 pipe (92% busy, about 180 operations a site at |omega| = 0.1): 0.113 ms at 24^4, where the
 // eigenvectors by Jacobi sweeps are thousands of operations.
 constexpr int kNoLimb = (int)0x80000000;
 template <int NT>
 __global__ void __launch_bounds__(NT) k_expi(const double *__restrict__ omega, int4 *__restrict__ Gq,
-                                            double *__restrict__ g_out, int64_t V) {
+                                            double *__restrict__ G, int64_t V) {
   const int64_t s = (int64_t)blockIdx.x * NT + threadIdx.x;
   if (s >= V) return;
   double w[8];
@@ -263,8 +263,8 @@ __global__ void __launch_bounds__(NT) k_expi(const double *__restrict__ omega, i
   for (int e = 0; e < 9; ++e) q[e] = to_clq(g.e[e], top);
 #pragma unroll
   for (int e = 0; e < 9; ++e) {
-    if (Gq) Gq[(int64_t)e * V + s] = lq_in_range(top) ? to_int4(q[e]) : make_int4(kNoLimb, 0, 0, 0);
-    if (g_out) reinterpret_cast<double2 *>(g_out)[s * 9 + e] = to_vec<double>(g.e[e]);
+    Gq[(int64_t)e * V + s] = lq_in_range(top) ? to_int4(q[e]) : make_int4(kNoLimb, 0, 0, 0);
+    if (G) st(G, (int64_t)e * V + s, g.e[e]);
   }
 }
 __device__ __forceinline__ cx<double> g_element(const int4 *Gq, int64_t idx) {

@@ -1854,17 +1854,19 @@ extern "C" lgf_status lgf_update(lgf_ctx *ctx, double *links, const double *g, i
 
 // ------------------------------ differentiable functional ------------------------------
 // Shared set-up of lgf_functional / lgf_functional_grad: the device pointers, and omega -> g in limb planes (in
-// the buffer of the double g).
+// the buffer of the double g) and, with planes, in doubles.
 constexpr int NT_GRAD = 128;
-static lgf_status prepare_functional(lgf_ctx *ctx, const double *links, const double *omega, const double **ldev,
-                                     const double **odev) {
+static lgf_status prepare_functional(lgf_ctx *ctx, const double *links, const double *omega, bool planes,
+                                     const double **ldev, const double **odev) {
   TRY(check_ctx(ctx));
   TRY(ensure_common(ctx));
   TRY(setup_precision<double>(ctx, ctx->s64));
   const int64_t V = ctx->V;
   TRY(input_ptr(ctx, links, (size_t)4 * V * 144, &ctx->staging, &ctx->staging_bytes, ldev));
   TRY(input_ptr(ctx, omega, (size_t)V * 64, &ctx->staging2, &ctx->staging2_bytes, odev));
-  k_expi<NT><<<grid1(V, NT), NT, 0, ctx->stream>>>(*odev, reinterpret_cast<int4 *>(ctx->s64.G), nullptr, V);
+  // (the planes of the working links, which these calls do not need, take the planes of g)
+  k_expi<NT><<<grid1(V, NT), NT, 0, ctx->stream>>>(*odev, reinterpret_cast<int4 *>(ctx->s64.G),
+                                                  planes ? ctx->s64.U : nullptr, V);
   CKL();
   ctx->loaded = false;  // the working fields were overwritten
   return LGF_OK;
@@ -1873,7 +1875,7 @@ static lgf_status prepare_functional(lgf_ctx *ctx, const double *links, const do
 extern "C" lgf_status lgf_functional(lgf_ctx *ctx, const double *links, const double *omega, double *F,
                                      double *g_out) {
   const double *ldev = nullptr, *odev = nullptr;
-  TRY(prepare_functional(ctx, links, omega, &ldev, &odev));
+  TRY(prepare_functional(ctx, links, omega, g_out != nullptr, &ldev, &odev));
   const int64_t V = ctx->V;
   memset(&ctx->ctrl_host, 0, sizeof(Ctrl));
   TRY(write_ctrl(ctx));
@@ -1884,8 +1886,7 @@ extern "C" lgf_status lgf_functional(lgf_ctx *ctx, const double *links, const do
     double *gdev = nullptr;
     bool host = false;
     TRY(output_ptr(ctx, g_out, (size_t)V * 144, &ctx->staging, &ctx->staging_bytes, &gdev, &host));
-    k_expi<NT><<<grid1(V, NT), NT, 0, ctx->stream>>>(odev, nullptr, gdev, V);
-    CKL();
+    TRY(from_planes<double>(ctx, ctx->s64.U, gdev, 1));  // omega has been read: g_out may lie over it
     if (host) CK(cudaMemcpyAsync(g_out, gdev, (size_t)V * 144, cudaMemcpyDeviceToHost, ctx->stream));
   }
   TRY(read_ctrl(ctx));
@@ -1896,17 +1897,22 @@ extern "C" lgf_status lgf_functional(lgf_ctx *ctx, const double *links, const do
 extern "C" lgf_status lgf_functional_grad(lgf_ctx *ctx, const double *links, const double *omega, double scale,
                                           double *grad) {
   const double *ldev = nullptr, *odev = nullptr;
-  TRY(prepare_functional(ctx, links, omega, &ldev, &odev));
+  TRY(prepare_functional(ctx, links, omega, false, &ldev, &odev));
   const int64_t V = ctx->V;
   double *gdev = nullptr;
   bool host = false;
-  // (a host gradient is gathered in the packed Delta buffer, which has its size and is not needed here)
+  // (a host gradient, or one that lies over what other threads still read, is gathered in the packed Delta
+  // buffer, which has its size and is not needed here; over omega itself each thread reads before it writes)
   double *packed = ctx->s64.P;
   size_t packed_bytes = (size_t)V * 64;
   TRY(output_ptr(ctx, grad, (size_t)V * 64, &packed, &packed_bytes, &gdev, &host));
+  const auto over = [&](const double *p, size_t per_site) { return gdev < p + per_site * V && p < gdev + (size_t)8 * V; };
+  const bool apart = !over(ldev, 72) && (gdev == odev || !over(odev, 8));
+  double *const out = apart ? gdev : ctx->s64.P;
   k_functional_grad<NT_GRAD><<<grid1(V, NT_GRAD), NT_GRAD, 0, ctx->stream>>>(
-      ldev, reinterpret_cast<const int4 *>(ctx->s64.G), odev, gdev, ctx->L, scale);
+      ldev, reinterpret_cast<const int4 *>(ctx->s64.G), odev, out, ctx->L, scale);
   CKL();
+  if (!apart) CK(cudaMemcpyAsync(gdev, out, packed_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
   if (host) CK(cudaMemcpyAsync(grad, gdev, (size_t)V * 64, cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   return LGF_OK;
