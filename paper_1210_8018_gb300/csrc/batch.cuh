@@ -13,17 +13,12 @@
 
 // ------------------------------------------------------------------------------------------------
 // FFT autotuner: candidates are the generic passes and the specialised passes with 16- or 32-wide
-// column tiles; each is timed on the context's own packed buffers and the fastest is kept. Results are
-// cached in a JSON object {"<Nx>x<Ny>x<Nz>x<Nt>:<f64|f32>": {"plan": "...", "C": c, "ms": t}, ...} at
+// column tiles; each is timed on the context's own packed buffers and the fastest is kept for the life of
+// the context (captured graphs hold its launches, whatever becomes of the cache file). Results are cached
+// in a JSON object {"<Nx>x<Ny>x<Nz>x<Nt>:<f64|f32>": {"plan": "...", "C": c, "ms": t}, ...} at
 // $LGF_TUNE_CACHE (default $HOME/.cache/lgf_fft_tune.json).
 // ------------------------------------------------------------------------------------------------
 namespace {
-
-struct TuneEntry {
-  std::string plan;  // "fixed" or "generic"
-  int C = 0;
-  double ms = 0;
-};
 
 std::string tune_cache_path() {
   const char *p = std::getenv("LGF_TUNE_CACHE");
@@ -87,6 +82,11 @@ template <typename T> std::string tune_key(const lgf_ctx *ctx) {
          std::to_string(ctx->n[3]) + (sizeof(T) == 8 ? ":f64" : ":f32");
 }
 
+template <typename T> std::string describe_plan(const lgf_ctx *ctx, const State<T> &S) {
+  return tune_key<T>(ctx) + "=" +
+         (S.tuned.plan.empty() ? "default" : S.tuned.plan + "/" + std::to_string(S.tuned.C)) + " ";
+}
+
 // Apply a candidate: re-plan the passes and opt the kernels in to their shared memory.
 template <typename T> lgf_status apply_fft_choice(lgf_ctx *ctx, State<T> &S, bool generic, int C) {
   ctx->generic_fft = generic;
@@ -121,13 +121,14 @@ template <typename T> lgf_status time_fft(lgf_ctx *ctx, State<T> &S, double *ms_
   return LGF_OK;
 }
 
-template <typename T> lgf_status autotune_fft(lgf_ctx *ctx, State<T> &S, TuneEntry *chosen) {
+template <typename T> lgf_status autotune_fft(lgf_ctx *ctx, State<T> &S) {
+  if (!S.tuned.plan.empty()) return LGF_OK;
   const std::string key = tune_key<T>(ctx);
   auto cache = tune_cache_read();
   auto it = cache.find(key);
   if (it != cache.end()) {
     TRY(apply_fft_choice<T>(ctx, S, it->second.plan == "generic", it->second.C));
-    *chosen = it->second;
+    S.tuned = it->second;
     return LGF_OK;
   }
   CK(cudaMemsetAsync(S.P, 0, sizeof(T) * 2 * 4 * (size_t)ctx->V * ctx->nb, ctx->stream));
@@ -154,7 +155,7 @@ template <typename T> lgf_status autotune_fft(lgf_ctx *ctx, State<T> &S, TuneEnt
   cache = tune_cache_read();
   cache[key] = best;
   tune_cache_write(cache);
-  *chosen = best;
+  S.tuned = best;
   return LGF_OK;
 }
 
@@ -411,9 +412,8 @@ lgf_status lgf_batch_fix(lgf_batch *b, double *const *links, double alpha, doubl
     BTRY(g, ensure_common(g));
     if (has_double) {
       BTRY(g, setup_precision<double>(g, g->s64));
-      TuneEntry e;
-      if (b->autotune) BTRY(g, autotune_fft<double>(g, g->s64, &e));
-      b->tuned[0] += tune_key<double>(g) + "=" + (b->autotune ? e.plan + "/" + std::to_string(e.C) : "default") + " ";
+      if (b->autotune) BTRY(g, autotune_fft<double>(g, g->s64));
+      b->tuned[0] += describe_plan<double>(g, g->s64);
     }
     if (has_float) {
       BTRY(g, setup_precision<float>(g, g->s32));
@@ -423,9 +423,8 @@ lgf_status lgf_batch_fix(lgf_batch *b, double *const *links, double alpha, doubl
         BTRY(g, alloc(g, &g->Rres, (size_t)g->nb * 72 * g->V));
         BTRY(g, alloc(g, &g->Kres, (size_t)g->nb * 18 * g->V));
       }
-      TuneEntry e;
-      if (b->autotune) BTRY(g, autotune_fft<float>(g, g->s32, &e));
-      b->tuned[1] += tune_key<float>(g) + "=" + (b->autotune ? e.plan + "/" + std::to_string(e.C) : "default") + " ";
+      if (b->autotune) BTRY(g, autotune_fft<float>(g, g->s32));
+      b->tuned[1] += describe_plan<float>(g, g->s32);
     }
   }
   for (int i = 0; i < b->n; ++i) {

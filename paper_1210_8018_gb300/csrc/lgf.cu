@@ -89,15 +89,23 @@ struct Pass {
 constexpr int kFixedThreads = 256;
 bool fixed_len(int n) { return n == 8 || n == 16 || n == 24 || n == 32 || n == 48 || n == 64; }
 
+// A choice of the FFT tuner (batch.cuh).
+struct TuneEntry {
+  std::string plan;  // "fixed" or "generic", empty where nothing has been chosen
+  int C = 0;
+  double ms = 0;
+};
+
 template <typename T> struct State {
   T *U = nullptr;  // links, planes
   T *P = nullptr;  // packed Delta / Delta-tilde, 4 planes
   T *G = nullptr;  // g, 9 planes
   float *A = nullptr;  // double path: a = g - 1 in double-float, 9 planes of float4
   void *tw[4] = {nullptr, nullptr, nullptr, nullptr};
-  void *weights = nullptr;  // filter weight of every site, when the plan's filter pass is a general one
+  void *weights = nullptr;  // filter weight of every site, once a plan's filter pass is a general one
   std::vector<Pass> passes;
   FFTTables tables;
+  TuneEntry tuned;  // in a batch: the plan of `passes`, chosen once (captured graphs hold its launches)
 };
 
 struct SiteGrid {
@@ -594,7 +602,8 @@ template <typename T> lgf_status opt_in_smem(lgf_ctx *ctx, State<T> &S) {
   });
 }
 
-// The weight table of a plan whose filter pass reads one (freed when the plan no longer does).
+// The weight table of a plan whose filter pass reads one. It stays until the context is destroyed: a graph that
+// was captured with such a plan holds its address.
 template <typename T> lgf_status ensure_weights(lgf_ctx *ctx, State<T> &S) {
   bool need = false;
   for (auto &p : S.passes) need |= p.kind == 0 && p.d.mode == 2;
@@ -608,10 +617,6 @@ template <typename T> lgf_status ensure_weights(lgf_ctx *ctx, State<T> &S) {
       return LGF_OK;
     }));
     CK(cudaStreamSynchronize(ctx->stream));  // later passes may run on another stream
-  } else if (!need && S.weights) {
-    CK(cudaStreamSynchronize(ctx->stream));
-    CK(cudaFree(S.weights));
-    S.weights = nullptr;
   }
   S.tables.weights = S.weights;
   return LGF_OK;
