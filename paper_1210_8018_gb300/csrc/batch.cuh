@@ -127,9 +127,9 @@ template <typename T> lgf_status autotune_fft(lgf_ctx *ctx, State<T> &S) {
   auto cache = tune_cache_read();
   auto it = cache.find(key);
   if (it != cache.end()) {
-    TRY(apply_fft_choice<T>(ctx, S, it->second.plan == "generic", it->second.C));
-    S.tuned = it->second;
-    return LGF_OK;
+    const lgf_status st = apply_fft_choice<T>(ctx, S, it->second.plan == "generic", it->second.C);
+    if (st == LGF_OK) S.tuned = it->second;
+    if (st != LGF_ENOMEM) return st;
   }
   CK(cudaMemsetAsync(S.P, 0, sizeof(T) * 2 * 4 * (size_t)ctx->V * ctx->nb, ctx->stream));
   struct Cand {
@@ -140,7 +140,9 @@ template <typename T> lgf_status autotune_fft(lgf_ctx *ctx, State<T> &S) {
   TuneEntry best;
   best.ms = 1e30;
   for (const Cand &c : cands) {
-    TRY(apply_fft_choice<T>(ctx, S, c.generic, c.C));
+    const lgf_status st = apply_fft_choice<T>(ctx, S, c.generic, c.C);
+    if (st == LGF_ENOMEM) continue;  // no room for the weight table of the general passes
+    TRY(st);
     const bool fixed_plan = !S.passes.empty() && S.passes[0].kind != 0;
     if (!c.generic && !fixed_plan) continue;  // the specialised passes do not fit this shape
     double ms = 0;
@@ -151,6 +153,7 @@ template <typename T> lgf_status autotune_fft(lgf_ctx *ctx, State<T> &S) {
       best.C = c.C;
     }
   }
+  if (best.plan.empty()) return LGF_ENOMEM;
   TRY(apply_fft_choice<T>(ctx, S, best.plan == "generic", best.C));
   cache = tune_cache_read();
   cache[key] = best;

@@ -105,6 +105,7 @@ template <typename T> struct State {
   void *weights = nullptr;  // filter weight of every site, once a plan's filter pass is a general one
   std::vector<Pass> passes;
   FFTTables tables;
+  bool ready = false;  // plan and tables are complete (set-up that ran out of memory is taken up again)
   TuneEntry tuned;  // in a batch: the plan of `passes`, chosen once (captured graphs hold its launches)
 };
 
@@ -208,6 +209,7 @@ lgf_status fail(lgf_ctx *c, lgf_status st, const std::string &msg) {
 #define CK(call)                                                                                    \
   do {                                                                                              \
     cudaError_t e_ = (call);                                                                        \
+    if (e_ == cudaErrorMemoryAllocation) cudaGetLastError(); /* not the next launch's error */      \
     if (e_ != cudaSuccess)                                                                          \
       return fail(ctx, e_ == cudaErrorMemoryAllocation ? LGF_ENOMEM : LGF_ECUDA,                    \
                   std::string(#call) + ": " + cudaGetErrorString(e_));                              \
@@ -629,8 +631,9 @@ template <typename T> lgf_status setup_precision(lgf_ctx *ctx, State<T> &S) {
   TRY(alloc(ctx, &S.P, nb * 4 * V * 2));
   TRY(alloc(ctx, &S.G, nb * 9 * V * 2));
   if constexpr (std::is_same<T, double>::value) TRY(alloc(ctx, &S.A, nb * 9 * V * 4));
-  if (!S.tw[0]) {
+  if (!S.ready) {
     for (int mu = 0; mu < 4; ++mu) {
+      if (S.tw[mu]) continue;
       const int N = ctx->n[mu];
       TRY(with_fft_type<T>(ctx, [&](auto tag) -> lgf_status {
         using FT = decltype(tag);
@@ -657,6 +660,7 @@ template <typename T> lgf_status setup_precision(lgf_ctx *ctx, State<T> &S) {
         CK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
       }
     }
+    S.ready = true;
   }
   return LGF_OK;
 }
