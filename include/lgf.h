@@ -195,8 +195,10 @@ lgf_status lgf_kernel_times(lgf_ctx *ctx, const char **name, long *launches, dou
  * Configurations of equal shape form a group whose kernels are launched once per group for all its
  * configurations; the iteration loop of all groups is captured in a CUDA graph and replayed until every
  * configuration has stopped (each keeps its own loop control, so iteration counts are per
- * configuration). FFT pass shapes are autotuned per (shape, precision) and cached in the JSON file
- * $LGF_TUNE_CACHE (default $HOME/.cache/lgf_fft_tune.json); LGF_AUTOTUNE=0 disables the tuner. ---- */
+ * configuration). FFT pass shapes are autotuned per group and precision by the first fix that needs them,
+ * stay for the life of the batch, and are cached per shape, precision, configurations of the group and GPU in
+ * the JSON file $LGF_TUNE_CACHE (default $HOME/.cache/lgf_fft_tune.json); LGF_AUTOTUNE=0 disables the
+ * tuner. ---- */
 typedef struct lgf_batch lgf_batch;
 
 /* dims: n x 4 extents (Nx, Ny, Nz, Nt), each as for lgf_create. */

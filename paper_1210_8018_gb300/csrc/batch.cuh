@@ -15,8 +15,9 @@
 // FFT autotuner: candidates are the generic passes and the specialised passes with 16- or 32-wide
 // column tiles; each is timed on the context's own packed buffers and the fastest is kept for the life of
 // the context (captured graphs hold its launches, whatever becomes of the cache file). Results are cached
-// in a JSON object {"<Nx>x<Ny>x<Nz>x<Nt>:<f64|f32>": {"plan": "...", "C": c, "ms": t}, ...} at
-// $LGF_TUNE_CACHE (default $HOME/.cache/lgf_fft_tune.json).
+// in a JSON object {"<key>": {"plan": "...", "C": c, "ms": t}, ...} at $LGF_TUNE_CACHE (default
+// $HOME/.cache/lgf_fft_tune.json). The key names all that the times depend on: extents, arithmetic,
+// configurations per launch, switches, GPU, and the version of the passes.
 // ------------------------------------------------------------------------------------------------
 namespace {
 
@@ -51,7 +52,8 @@ std::map<std::string, TuneEntry> tune_cache_read() {
     char plan[32] = {0};
     if (std::sscanf(body.c_str(), "{\"plan\": \"%31[a-z]\", \"C\": %d, \"ms\": %lf}", plan, &e.C, &e.ms) == 3) {
       e.plan = plan;
-      m[key] = e;
+      // (there are no kernels for other widths)
+      if (e.plan == "generic" || (e.plan == "fixed" && (e.C == 16 || e.C == 32))) m[key] = e;
     }
     pos = close + 1;
   }
@@ -77,13 +79,27 @@ void tune_cache_write(const std::map<std::string, TuneEntry> &m) {
   std::rename(tmp.c_str(), path.c_str());
 }
 
-template <typename T> std::string tune_key(const lgf_ctx *ctx) {
+constexpr int kFftVersion = 2;  // to be raised with every change of the passes or of their plans
+
+template <typename T> std::string plan_label(const lgf_ctx *ctx) {
   return std::to_string(ctx->n[0]) + "x" + std::to_string(ctx->n[1]) + "x" + std::to_string(ctx->n[2]) + "x" +
          std::to_string(ctx->n[3]) + (sizeof(T) == 8 ? ":f64" : ":f32");
 }
 
+template <typename T> std::string tune_key(const lgf_ctx *ctx) {
+  cudaDeviceProp prop;
+  std::string gpu = cudaGetDeviceProperties(&prop, ctx->device) == cudaSuccess ? prop.name : "unknown";
+  for (char &c : gpu)
+    if (c == '"' || c == '\\' || c == '{' || c == '}') c = ' ';
+  const bool f64 = sizeof(T) == 8;
+  return plan_label<T>(ctx) + (f64 ? (ctx->fft_df64 ? ":df64" : ":double") : ":float") + ":nb" +
+         std::to_string(ctx->nb) + ":zt" + std::to_string(ctx->fft_zt) + "xy" + std::to_string(ctx->xy_reg) + "tf" +
+         std::to_string(ctx->tfilter_reg) + "p" + std::to_string(ctx->fft_persist) + ":" + gpu + ":v" +
+         std::to_string(kFftVersion);
+}
+
 template <typename T> std::string describe_plan(const lgf_ctx *ctx, const State<T> &S) {
-  return tune_key<T>(ctx) + "=" +
+  return plan_label<T>(ctx) + "=" +
          (S.tuned.plan.empty() ? "default" : S.tuned.plan + "/" + std::to_string(S.tuned.C)) + " ";
 }
 
