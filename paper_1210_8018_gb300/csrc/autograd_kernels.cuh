@@ -107,11 +107,10 @@ __device__ __forceinline__ void expi_from_eig(const m3<double> &W, const double 
 }
 
 // Hermitian matrix with diagonal d and upper elements 01, 02, 12.
-template <typename T> struct herm_of {
-  T d[3];
-  cx<T> a, b, c;
+struct herm {
+  double d[3];
+  cx<double> a, b, c;
 };
-using herm = herm_of<double>;
 __device__ __forceinline__ herm algebra_herm(const double w[8], double scale) {
   const double s3 = 0.57735026918962576451, h = 0.5 * scale;  // 1/sqrt(3)
   return {{h * fma(s3, w[7], w[2]), h * fma(s3, w[7], -w[2]), -2.0 * h * s3 * w[7]},
@@ -126,7 +125,7 @@ __device__ __forceinline__ double algebra_norm2(const double w[8]) {
   for (int a = 0; a < 8; ++a) t = fma(w[a], w[a], t);
   return 0.5 * t;
 }
-// Norm 3 (m <= 4): below it the gradient's error is smaller than by eigenvectors (rms 2.2e-16 of the gradient against
+// Norm 3 (m <= 3): below it the gradient's error is smaller than by eigenvectors (rms 2.2e-16 of the gradient against
 // 1.0e-15 at |omega| = 0.1, 8.7e-16 against 1.2e-15 at 2), at a norm of 10 the doublings have made it larger.
 constexpr double kSeriesNorm2 = 9.0;
 __device__ __forceinline__ int halvings(double norm2) {
@@ -398,39 +397,35 @@ __device__ __noinline__ void gradient_by_eigenvectors(const double *w, const m3<
 }
 
 // D A = -i [H, A]
-template <typename T> __device__ __forceinline__ herm_of<T> commutator(const herm_of<T> &h, const herm_of<T> &x) {
-  auto minus_i = [](cx<T> v) { return cx<T>{v.i, -v.r}; };
-  auto off = [&](cx<T> z, T dh, T dx, cx<T> hz) {  // dh z - hz dx
-    return cx<T>{fma(dh, z.r, -dx * hz.r), fma(dh, z.i, -dx * hz.i)};
+__device__ __forceinline__ herm commutator(const herm &h, const herm &x) {
+  auto minus_i = [](cx<double> v) { return cx<double>{v.i, -v.r}; };
+  auto off = [&](cx<double> z, double dh, double dx, cx<double> hz) {  // dh z - hz dx
+    return cx<double>{fma(dh, z.r, -dx * hz.r), fma(dh, z.i, -dx * hz.i)};
   };
-  herm_of<T> y;
-  cx<T> t = off(x.a, h.d[0] - h.d[1], x.d[0] - x.d[1], h.a);
+  herm y;
+  cx<double> t = off(x.a, h.d[0] - h.d[1], x.d[0] - x.d[1], h.a);
   t = cmac_cj(t, h.b, x.c);
-  y.a = minus_i(cmac_cj(t, cx<T>{-x.b.r, -x.b.i}, h.c));
+  y.a = minus_i(cmac_cj(t, cx<double>{-x.b.r, -x.b.i}, h.c));
   t = off(x.b, h.d[0] - h.d[2], x.d[0] - x.d[2], h.b);
   t = cmac(t, h.a, x.c);
-  y.b = minus_i(cmac(t, cx<T>{-h.c.r, -h.c.i}, x.a));
+  y.b = minus_i(cmac(t, cx<double>{-h.c.r, -h.c.i}, x.a));
   t = off(x.c, h.d[1] - h.d[2], x.d[1] - x.d[2], h.c);
   t = cmac_cj(t, x.b, h.a);
-  y.c = minus_i(cmac_cj(t, cx<T>{-h.b.r, -h.b.i}, x.a));
+  y.c = minus_i(cmac_cj(t, cx<double>{-h.b.r, -h.b.i}, x.a));
   // 2 Im of the diagonal of H A
-  const T ia = fma(h.a.i, x.a.r, -h.a.r * x.a.i), ib = fma(h.b.i, x.b.r, -h.b.r * x.b.i);
-  const T ic = fma(h.c.i, x.c.r, -h.c.r * x.c.i);
+  const double ia = fma(h.a.i, x.a.r, -h.a.r * x.a.i), ib = fma(h.b.i, x.b.r, -h.b.r * x.b.i);
+  const double ic = fma(h.c.i, x.c.r, -h.c.r * x.c.i);
   y.d[0] = 2 * (ia + ib);
   y.d[1] = 2 * (ic - ia);
   y.d[2] = -2 * (ib + ic);
   return y;
 }
-template <typename T> __device__ __forceinline__ void herm_axpy(herm_of<T> &y, T s, const herm_of<T> &x) {
+__device__ __forceinline__ void herm_axpy(herm &y, double s, const herm &x) {
 #pragma unroll
   for (int i = 0; i < 3; ++i) y.d[i] = fma(s, x.d[i], y.d[i]);
   y.a = {fma(s, x.a.r, y.a.r), fma(s, x.a.i, y.a.i)};
   y.b = {fma(s, x.b.r, y.b.r), fma(s, x.b.i, y.b.i)};
   y.c = {fma(s, x.c.r, y.c.r), fma(s, x.c.i, y.c.i)};
-}
-template <typename D, typename S> __device__ __forceinline__ herm_of<D> herm_cast(const herm_of<S> &x) {
-  auto c = [](cx<S> v) { return cx<D>{(D)v.r, (D)v.i}; };
-  return {{(D)x.d[0], (D)x.d[1], (D)x.d[2]}, c(x.a), c(x.b), c(x.c)};
 }
 // Y <- (Y + g^+ Y g) / 2
 __device__ __noinline__ void conjugate_average(herm *y, const m3<double> *g) {
@@ -459,9 +454,10 @@ __device__ __noinline__ void conjugate_average(herm *y, const m3<double> *g) {
 
 // dF/d omega^a(x), a = 0..7, written site-major (V x 8), scaled by `scale` (the incoming gradient). U: the
 // caller's links; g in limb planes. The staple is summed in 59 fractional bits (its elements reach 8).
-// Bound by the FP64 pipe: with all eleven terms of the series in double (570 of 900 operations at |omega| = 0.1) 0.64 ms
-// at 24^4, the pipe 87% busy. A step of gradient-based fixing (F, gradient, Fourier filter) took 5.40 ms with Jacobi
-// eigenvectors and FP64 products in both calls, 1.58 with the series in double, and takes 1.45 ms.
+// Bound by the FP64 pipe (87% busy, 570 of 900 operations in the eleven terms of the series at |omega| = 0.1): 0.64 ms
+// at 24^4. A step of gradient-based fixing (F, gradient, Fourier filter) took 5.40 ms with Jacobi eigenvectors and FP64
+// products in both calls, and takes 1.55 ms. (The terms below 2^-34 of the sum in float would make it 1.44, with
+// those of links beyond 1e38 infinite.)
 template <int NT>
 __global__ void __launch_bounds__(NT, 3) k_functional_grad(const double *__restrict__ U, const int4 *__restrict__ Gq,
                                                        const double *omega, double *grad, Lattice L, double scale) {
@@ -579,26 +575,12 @@ __global__ void __launch_bounds__(NT, 3) k_functional_grad(const double *__restr
     herm y = x;
     const float z = 1.41422f * norm;  // bounds |ad_H|: its eigenvalues are differences of those of H
     float term = 1.f;
-    int n = 1;
 #pragma unroll 1
-    for (; n < 19; ++n) {  // z < 0.71: the 18th term is below 1e-18 of the sum
+    for (int n = 1; n < 19; ++n) {  // z < 0.71: the 18th term is below 1e-18 of the sum
       x = commutator(h, x);
       herm_axpy(y, fabs(kExpCoef[n + 1]), x);
       term *= z / (float)(n + 1);  // z^n / (n+1)!
-      if (term < 0x1p-34f) break;
-    }
-    if (n < 18 && term >= 1e-17f) {
-      // the terms below 2^-34 of the sum need no more than float: their rounding is below 2^-58 of it
-      const herm_of<float> hf = herm_cast<float>(h);
-      herm_of<float> xf = herm_cast<float>(x), yf = {};
-#pragma unroll 1
-      for (++n; n < 19; ++n) {
-        xf = commutator(hf, xf);
-        herm_axpy(yf, (float)fabs(kExpCoef[n + 1]), xf);
-        term *= z / (float)(n + 1);
-        if (term < 1e-17f) break;
-      }
-      herm_axpy(y, 1.0, herm_cast<double>(yf));
+      if (term < 1e-17f) break;
     }
     if (m > 0) {
       exp_poly p = exp_series(h, norm);
