@@ -19,7 +19,8 @@
 // W^+, Daleckii-Krein: W (Phi o (W^+ K W)) W^+ with Phi_jk = exp(i (l_j + l_k)/2) sinc((l_j - l_k)/2)).
 //
 // Products with O(1) matrices (g U, the staple) run in 60-bit fixed point (q60.cuh); a site that meets a link
-// which is not near SU(3) forms them in FP64.
+// which is not near SU(3) forms them in FP64, and so does the staple of a site around which all matrices have the
+// same elements close to zero (part_check), the gradient of which may be as small.
 #pragma once
 #include "site_kernels.cuh"
 
@@ -346,8 +347,8 @@ __device__ __forceinline__ double sinc_half(double x) {  // sin(x)/x
   return sin(x) / x;
 }
 
-// The staple K(x) in FP64, for links out of the fixed-point range.
-__device__ __noinline__ void staple_fp64(const double2 *U, const int4 *Gq, const Lattice *L, int64_t s, const int *c,
+// The staple K(x) in FP64, for fields that are not for the fixed point. g in planes.
+__device__ __noinline__ void staple_fp64(const double2 *U, const double *G, const Lattice *L, int64_t s, const int *c,
                                          m3<double> *K) {
   const int64_t V = L->V;
   for (int e = 0; e < 9; ++e) K->e[e] = {0, 0};
@@ -358,8 +359,8 @@ __device__ __noinline__ void staple_fp64(const double2 *U, const int4 *Gq, const
       for (int j = 0; j < 3; ++j) {
         cx<double> t = K->e[3 * i + j], b = {0, 0};
         for (int k = 0; k < 3; ++k) {
-          t = cmac_cj(t, from_vec<double>(u[3 * i + k]), g_element(Gq, (int64_t)(3 * j + k) * V + sf));
-          b = cmac(b, g_element(Gq, (int64_t)(3 * j + k) * V + sb), from_vec<double>(ub[3 * k + i]));
+          t = cmac_cj(t, from_vec<double>(u[3 * i + k]), ldg(G, (int64_t)(3 * j + k) * V + sf));
+          b = cmac(b, ldg(G, (int64_t)(3 * j + k) * V + sb), from_vec<double>(ub[3 * k + i]));
         }
         K->e[3 * i + j] = t + conjg(b);
       }
@@ -453,14 +454,14 @@ __device__ __noinline__ void conjugate_average(herm *y, const m3<double> *g) {
 }
 
 // dF/d omega^a(x), a = 0..7, written site-major (V x 8), scaled by `scale` (the incoming gradient). U: the
-// caller's links; g in limb planes. The staple is summed in 59 fractional bits (its elements reach 8).
+// caller's links; g in limb planes and in planes of doubles. The staple is summed in 59 fractional bits (its elements reach 8).
 // Bound by the FP64 pipe (87% busy, 570 of 900 operations in the eleven terms of the series at |omega| = 0.1): 0.64 ms
 // at 24^4. A step of gradient-based fixing (F, gradient, Fourier filter) took 5.40 ms with Jacobi eigenvectors and FP64
-// products in both calls, and takes 1.55 ms. (The terms below 2^-34 of the sum in float would make it 1.44, with
+// products in both calls, and takes 1.57 ms (1.55 without part_check). (The terms below 2^-34 of the sum in float would make it 1.44, with
 // those of links beyond 1e38 infinite.)
 template <int NT>
 __global__ void __launch_bounds__(NT, 3) k_functional_grad(const double *__restrict__ U, const int4 *__restrict__ Gq,
-                                                       const double *omega, double *grad, Lattice L, double scale) {
+                                                       const double *__restrict__ G, const double *omega, double *grad, Lattice L, double scale) {
   const int64_t V = L.V;
   const int64_t s = (int64_t)blockIdx.x * NT + threadIdx.x;
   if (s >= V) return;
@@ -471,6 +472,7 @@ __global__ void __launch_bounds__(NT, 3) k_functional_grad(const double *__restr
   {
     long long kr[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, ki[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     bool bad = false;
+    part_check parts;
 #pragma unroll 1
     for (int mu = 0; mu < 4; ++mu) {
       const int64_t sf = site_fwd(L, s, mu, c[mu]), sb = site_back(L, s, mu, c[mu]);
@@ -489,6 +491,7 @@ __global__ void __launch_bounds__(NT, 3) k_functional_grad(const double *__restr
           for (int k = 0; k < 3; ++k) {
             const clq x = to_clq(from_vec<double>(__ldg(u + 3 * i + k)), top);
             unit.add(i, k, x);
+            parts.add(i, k, x);
 #pragma unroll
             for (int j = 0; j < 3; ++j) clmac_cj(t[j], x, g[3 * j + k]);
           }
@@ -515,6 +518,7 @@ __global__ void __launch_bounds__(NT, 3) k_functional_grad(const double *__restr
           for (int k = 0; k < 3; ++k) {
             const clq x = to_clq(from_vec<double>(__ldg(u + 3 * k + i)), top);
             unit.add(k, i, x);
+            parts.add(k, i, x);
 #pragma unroll
             for (int j = 0; j < 3; ++j) clmac(t[j], g[3 * j + k], x);
           }
@@ -527,10 +531,12 @@ __global__ void __launch_bounds__(NT, 3) k_functional_grad(const double *__restr
         bad |= !unit.ok(top);
       }
     }
-    if (bad) {
+#pragma unroll
+    for (int e = 0; e < 9; ++e) parts.add(e / 3, e % 3, ldg_q(Gq, (int64_t)e * V + s));
+    if (bad || parts.small()) {
       m3<double> t;
       const Lattice Lc = L;
-      staple_fp64(U2, Gq, &Lc, s, c, &t);
+      staple_fp64(U2, G, &Lc, s, c, &t);
       K = t;
     } else {
 #pragma unroll
@@ -557,7 +563,7 @@ __global__ void __launch_bounds__(NT, 3) k_functional_grad(const double *__restr
         for (int j = 0; j < 3; ++j) M[3 * i + j] = {0, 0};
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          const cx<double> g = g_element(Gq, (int64_t)(3 * i + k) * V + s);
+          const cx<double> g = ldg(G, (int64_t)(3 * i + k) * V + s);
 #pragma unroll
           for (int j = 0; j < 3; ++j) {
             if (i != j) M[3 * i + j] = cmac(M[3 * i + j], g, K.e[3 * k + j]);

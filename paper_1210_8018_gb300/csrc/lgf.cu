@@ -1906,7 +1906,7 @@ extern "C" lgf_status lgf_functional(lgf_ctx *ctx, const double *links, const do
 extern "C" lgf_status lgf_functional_grad(lgf_ctx *ctx, const double *links, const double *omega, double scale,
                                           double *grad) {
   const double *ldev = nullptr, *odev = nullptr;
-  TRY(prepare_functional(ctx, links, omega, false, &ldev, &odev));
+  TRY(prepare_functional(ctx, links, omega, true, &ldev, &odev));
   const int64_t V = ctx->V;
   double *gdev = nullptr;
   bool host = false;
@@ -1919,7 +1919,7 @@ extern "C" lgf_status lgf_functional_grad(lgf_ctx *ctx, const double *links, con
   const bool apart = !over(ldev, 72) && (gdev == odev || !over(odev, 8));
   double *const out = apart ? gdev : ctx->s64.P;
   k_functional_grad<NT_GRAD><<<grid1(V, NT_GRAD), NT_GRAD, 0, ctx->stream>>>(
-      ldev, reinterpret_cast<const int4 *>(ctx->s64.G), odev, out, ctx->L, scale);
+      ldev, reinterpret_cast<const int4 *>(ctx->s64.G), ctx->s64.U, odev, out, ctx->L, scale);
   CKL();
   if (!apart) CK(cudaMemcpyAsync(gdev, out, packed_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
   if (host) CK(cudaMemcpyAsync(grad, gdev, (size_t)V * 64, cudaMemcpyDeviceToHost, ctx->stream));

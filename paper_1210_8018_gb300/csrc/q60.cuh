@@ -64,19 +64,39 @@ __device__ __forceinline__ clq ldg_q(const int4 *p, int64_t idx) {
 __device__ __forceinline__ int4 to_int4(clq a) { return make_int4(a.r.h, a.r.l, a.i.h, a.i.l); }
 __device__ __forceinline__ double lq_double(lq a) { return q60_double(lq_join(a)); }
 
-// Rows and columns of at most unit length (to 1.5%): the products of such matrices, and their sums, stay in
-// range whatever the entries are. Gathered one element at a time (|x| < 2 each: 14-bit squares, 31-bit sums).
+// Rows and columns of about unit length: at most (to 1.5%), so that the products of such matrices, and their sums,
+// stay in range whatever the entries are, and at least a quarter, because FP64 products of shorter ones would err by
+// less than 2^-57. Gathered one element at a time (|x| < 2 each: 14-bit squares, 31-bit sums).
 struct unit_check {
   int row[3] = {0, 0, 0}, col[3] = {0, 0, 0};
+  __device__ static __forceinline__ int square(clq a) {
+    const int x = a.r.h >> 17, y = a.i.h >> 17;
+    return x * x + y * y;
+  }
   __device__ __forceinline__ void add(int i, int j, clq a) {
-    const int x = a.r.h >> 17, y = a.i.h >> 17, n = x * x + y * y;
+    const int n = square(a);
     row[i] += n;
     col[j] += n;
   }
   __device__ __forceinline__ bool ok(unsigned top) const {
-    constexpr int limit = 69000000;  // 2^26 is a unit vector
+    constexpr int most = 69000000, least = 1 << 22;  // 2^26 is a unit vector
     return lq_in_range(top) &&
-           max(max(max(row[0], row[1]), row[2]), max(max(col[0], col[1]), col[2])) <= limit;
+           max(max(max(row[0], row[1]), row[2]), max(max(col[0], col[1]), col[2])) <= most &&
+           min(min(min(row[0], row[1]), row[2]), min(min(col[0], col[1]), col[2])) >= least;
+  }
+};
+
+// The elements by their part in an anti-Hermitian matrix, over all the matrices that enter a sum: the three pairs
+// beside the diagonal and the three imaginary parts on it. Where the elements of one of them are all small, as those
+// of fields close to unity are, its 2^-60 would be more than the rounding of FP64.
+struct part_check {
+  int pair[3] = {0, 0, 0}, diag[3] = {0, 0, 0};
+  __device__ __forceinline__ void add(int i, int j, clq a) {
+    if (i == j) diag[i] |= (a.i.h >> 17) * (a.i.h >> 17);
+    else pair[i + j - 1] |= unit_check::square(a);
+  }
+  __device__ __forceinline__ bool small() const {  // all below 2^-5
+    return min(min(min(pair[0], pair[1]), pair[2]), min(min(diag[0], diag[1]), diag[2])) < (1 << 16);
   }
 };
 

@@ -1,5 +1,6 @@
-"""The gradient of the functional against extended precision: links far beyond the range of a float, and the norms
-of omega at which its series are doubled or left for the eigenvectors."""
+"""The gradient of the functional against extended precision where the 60-bit fixed point and the series could hold
+less than FP64: fields close to unity, links far from unit length, and the norms of omega at which the series are
+doubled or left for the eigenvectors."""
 import numpy as np
 import pytest
 
@@ -52,7 +53,39 @@ def device_gradient(U, w):
     return out
 
 
-@pytest.mark.parametrize("factor", [2.0 ** 135, 2.0 ** 500])
+def near_unity(d, seed):
+    rng = np.random.default_rng(seed)
+    x = d * (rng.normal(size=(4, SITES, 3, 3)) + 1j * rng.normal(size=(4, SITES, 3, 3)))
+    return np.ascontiguousarray((np.eye(3) + x - dag(x)).reshape((4,) + DIMS[::-1] + (3, 3))), rng
+
+
+# eight terms of size d to an element of the staple and three to one of M, whose rounding is that of their size:
+# fewer than 64 roundings of 16 d, over 12 V
+@pytest.mark.parametrize("omega", [0.0, 1.0])
+@pytest.mark.parametrize("d", [1e-12, 1e-9, 1e-6, 1e-3])
+def test_near_unity(d, omega):
+    U, rng = near_unity(d, 61)
+    w = omega * d * rng.normal(size=(SITES, 8))
+    err = np.abs(device_gradient(U, w) - gradient(U, w)).max()
+    assert err < 64 * 2.0 ** -53 * 16 * d / (12 * SITES), err
+
+
+def test_one_pair_of_elements_small():
+    """Links of an SU(2) subgroup, and the elements that leave it of size 1e-9."""
+    U, rng = near_unity(1e-9, 63)
+    a = rng.uniform(-3, 3, size=U.shape[:5])
+    c, s = np.cos(a), np.sin(a)
+    R = np.broadcast_to(np.eye(3, dtype=complex), U.shape).copy()
+    R[..., 0, 0], R[..., 0, 1], R[..., 1, 0], R[..., 1, 1] = c, s, -s, c
+    U = R @ U
+    U[..., 0, 0] *= np.exp(0.3j)
+    w = np.zeros((SITES, 8))
+    got, ref = device_gradient(U, w), gradient(U, w)
+    assert np.abs(got - ref)[:, 3:7].max() < 64 * 2.0 ** -53 * 16e-9 / (12 * SITES)
+    assert np.abs(got - ref).max() < 64 * 2.0 ** -53 * 16 / (12 * SITES)
+
+
+@pytest.mark.parametrize("factor", [2.0 ** -100, 2.0 ** 135, 2.0 ** 500])
 def test_scaled_links(factor):
     U = synth.config(DIMS, 65, 0.6)
     w = 0.1 * np.random.default_rng(66).normal(size=(SITES, 8))
