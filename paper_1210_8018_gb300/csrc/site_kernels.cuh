@@ -1204,7 +1204,8 @@ __global__ void __launch_bounds__(NT, 2) k_measure_q60(const int4 *__restrict__ 
     site_coords(L, s, c);
     {
       long long acc[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, tr = 0;
-      auto q56 = [](lq a) { return ((long long)a.h << 26) + (a.l >> 4); };
+      // towards zero (to_lq gives both limbs the number's sign), as k_delta converts
+      auto q56 = [](lq a) { return ((long long)a.h << 26) + a.l / 16; };
 #pragma unroll 1
       for (int mu = 0; mu < 4; ++mu) {
         const int4 *plane = Q + (int64_t)mu * 9 * V;

@@ -1,11 +1,11 @@
-"""The gradient of the functional against extended precision where the 60-bit fixed point and the series could hold
-less than FP64: fields close to unity, links far from unit length, and the norms of omega at which the series are
-doubled or left for the eigenvectors."""
+"""The gradient of the functional and the measurements against extended precision where the 60-bit fixed point and
+the series could hold less than FP64: fields close to unity, links far from unit length or between the steps of the
+fixed point, and the norms of omega at which the series are doubled or left for the eigenvectors."""
 import numpy as np
 import pytest
 
 import synth
-from helpers import gell_mann
+from helpers import gell_mann, identity_links
 
 pytestmark = pytest.mark.gpu
 
@@ -102,3 +102,30 @@ def test_norms_beside_the_rules(norm):
     w *= 2 ** 0.5 * norm / np.linalg.norm(w, axis=1, keepdims=True)
     err = np.abs(device_gradient(U, w) - gradient(U, w)).max()
     assert err < 64 * 2.0 ** -53 * 16 * (1 + norm) / (12 * SITES), err
+
+
+def test_measure_between_the_steps():
+    """Elements below the last step of Delta's fixed point are dropped whatever their sign, as lgf_delta drops them."""
+    import paper_1210_8018_gb300 as lgf
+    U = identity_links(DIMS)
+    U[1, 0, 1, 2, 3, 0, 1] = -2.0 ** -58
+    U[2, 1, 0, 1, 2, 1, 1] += -1j * 2.0 ** -58
+    with lgf.Lattice(DIMS) as lat:
+        theta, _ = lat.delta(U, np.empty(U.shape[1:], complex))
+        r = lat.measure(U)
+    assert r["theta"] == theta == 0.0
+    U = synth.config(DIMS, 69, 0.6)
+    with lgf.Lattice(DIMS) as lat:
+        theta, _ = lat.delta(U, np.empty(U.shape[1:], complex))
+        r = lat.measure(U)
+    assert abs(r["theta"] - theta) < 16 * 2.0 ** -53 * theta
+
+
+def test_measure_of_short_links():
+    import paper_1210_8018_gb300 as lgf
+    U = synth.config(DIMS, 70, 0.6)
+    with lgf.Lattice(DIMS) as lat:
+        r, q = lat.measure(U), lat.measure(U * 2.0 ** -100)
+    # nine terms to a product, four products, and their sum over the lattice
+    assert abs(q["plaquette"] * 2.0 ** 400 - r["plaquette"]) < 64 * 2.0 ** -53
+    assert abs(q["F"] * 2.0 ** 100 - r["F"]) < 64 * 2.0 ** -53
