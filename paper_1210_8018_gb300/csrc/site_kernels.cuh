@@ -1194,6 +1194,7 @@ __global__ void __launch_bounds__(NT) k_links_to_q60(const double *__restrict__ 
 template <int NT>
 __global__ void __launch_bounds__(NT, 2) k_measure_q60(const int4 *__restrict__ Q, double *partials, double *plaq_part,
                                                       Ctrl *ctrl, Lattice L, int spt, int with_plaq) {
+  if (ctrl->out_of_range) return;  // the FP64 kernels will do it
   const int64_t V = L.V;
   double th = 0.0, f = 0.0, pl = 0.0;
 #pragma unroll 1
