@@ -17,7 +17,9 @@
 // the context (captured graphs hold its launches, whatever becomes of the cache file). Results are cached
 // in a JSON object {"<key>": {"plan": "...", "C": c, "ms": t}, ...} at $LGF_TUNE_CACHE (default
 // $HOME/.cache/lgf_fft_tune.json). The key names all that the times depend on: extents, arithmetic,
-// configurations per launch, switches, GPU, and the version of the passes.
+// configurations per launch, GPU, and the version of the passes. (Contexts that differ only in the switches between
+// forms of the fixed-length passes, which give the same bits, share an entry: the general passes round differently,
+// and a comparison of two forms has to keep to one family.)
 // ------------------------------------------------------------------------------------------------
 namespace {
 
@@ -93,9 +95,7 @@ template <typename T> std::string tune_key(const lgf_ctx *ctx) {
     if (c == '"' || c == '\\' || c == '{' || c == '}') c = ' ';
   const bool f64 = sizeof(T) == 8;
   return plan_label<T>(ctx) + (f64 ? (ctx->fft_df64 ? ":df64" : ":double") : ":float") + ":nb" +
-         std::to_string(ctx->nb) + ":zt" + std::to_string(ctx->fft_zt) + "xy" + std::to_string(ctx->xy_reg) + "tf" +
-         std::to_string(ctx->tfilter_reg) + "p" + std::to_string(ctx->fft_persist) + ":" + gpu + ":v" +
-         std::to_string(kFftVersion);
+         std::to_string(ctx->nb) + ":" + gpu + ":v" + std::to_string(kFftVersion);
 }
 
 template <typename T> std::string describe_plan(const lgf_ctx *ctx, const State<T> &S) {
