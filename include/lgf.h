@@ -90,7 +90,14 @@ void lgf_default_options(lgf_options *opt);
  * the residual stage (float iterations on U = U_h + R, with R the float change since the handover, then
  * the double links rebuilt exactly). With LGF_REUNIT_FP64=1, LGF_RESIDUAL=0 and theta_switch = 1e-8
  * the mixed schedule is: float iterations with double reductions and periodic double reprojection until
- * theta <= 1e-8, the handover, and double iterations to theta < eps. */
+ * theta <= 1e-8, the handover, and double iterations to theta < eps.
+ * Further switches between forms of the same step: LGF_UPDATE_SPLIT=ab and LGF_HANDOVER_SPLIT=ab (two digits 0-4)
+ * give the links per site that the large-step double update and the handover form in FP64 in even and in odd
+ * warps, the others in fixed point (defaults 00 and 22; the same to FP64 rounding); and, with the same bits either
+ * way, LGF_FFT_ZT=0 (z, the filter on t, and z again as three FFT passes instead of one), LGF_TFILTER_REG=0 and
+ * LGF_XY_REG=0 (64-point FFT passes in shared memory instead of registers), LGF_FFT_PERSIST=0 (one FFT tile per
+ * block), LGF_TWALK=0 and LGF_TWALK_MIN_BLOCKS=n (site kernels in site order instead of walking along t, and the
+ * launch size from which they walk), LGF_PDL=0 (ordinary launches instead of programmatic stream serialisation). */
 lgf_status lgf_create(int Nx, int Ny, int Nz, int Nt, lgf_ctx **out);
 
 /* Release every resource of the context (NULL is accepted). */

@@ -58,9 +58,10 @@ template <typename T> __device__ __forceinline__ typename vec2<T>::type to_vec(c
 }
 template <> __device__ __forceinline__ float4 to_vec<df64>(cx<df64> a) { return make_float4(a.r.hi, a.r.lo, a.i.hi, a.i.lo); }
 
-// Global load of a vector in the order of the program: fields that another kernel of the iteration may have
-// written after this one was placed on the chip (follow_on) are not read-only for its lifetime, which the
-// non-coherent __ldg takes for granted, and nothing moves a volatile load to before the wait.
+// Coherent global load of a vector, in the order of the other volatile assembly: fields that another kernel of the
+// iteration may have written after this one was placed on the chip (follow_on) are not read-only for its lifetime,
+// which the non-coherent __ldg takes for granted, and no volatile load moves to before the wait. It is not ordered
+// against plain stores: a kernel that reads with it what the same thread has written needs more than this.
 __device__ __forceinline__ float2 ldv(const float2 *p) {
   float2 v;
   asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
