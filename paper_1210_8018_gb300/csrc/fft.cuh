@@ -65,6 +65,7 @@ struct PassDesc {
 };
 
 struct FFTTables {
+  AxisFFT ax[4];
   const void *tw[4];        // per lattice axis: N complex twiddles w_N^j (T)
   const double *p2part[4];  // per lattice axis: 4 sin^2(pi k(pos)/N) for the frequency at position pos
   double wscale;            // p^2_max / V

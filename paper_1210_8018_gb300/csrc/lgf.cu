@@ -646,6 +646,7 @@ template <typename T> lgf_status setup_precision(lgf_ctx *ctx, State<T> &S) {
     }
     plan_passes<T>(ctx, S);
     for (int mu = 0; mu < 4; ++mu) {
+      S.tables.ax[mu] = ctx->ax[mu];
       S.tables.tw[mu] = S.tw[mu];
       S.tables.p2part[mu] = ctx->p2part[mu];
       S.tables.n[mu] = ctx->n[mu];
