@@ -4,10 +4,9 @@
 namespace lgf {
 ZtKernel fft_df64_zt_long(int nz, int nt) {
   switch (nz) {
-    case 24: return zt_by_nt<df64, 24>(nt);
     case 32: return zt_by_nt<df64, 32>(nt);
-    case 48: return zt_by_nt<df64, 48>(nt);
-    default: return zt_by_nt<df64, 64>(nt);
+    case 64: return zt_by_nt<df64, 64>(nt);
+    default: return {};  // 24 and 48: none is faster (zt_faster)
   }
 }
 }  // namespace lgf
