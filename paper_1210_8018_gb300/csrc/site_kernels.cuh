@@ -780,10 +780,10 @@ __device__ __forceinline__ void update_link_small(double *plane, int64_t V, int6
 // stay below 6^(1/2) (1.76 + 1.01) = 6.8 of 8 (times 2^60). In row 2 they stay below 2 (1.76 + 1.76) = 7.1 for a
 // unitary g, which k_gauge's is; the caller's (AOS) is not checked for its angles, so there the two products'
 // cross sums, 5.1 each, are kept apart. And no less than FP64 would hold: no row of g or column of U shorter than
-// 1/4, not both U and g(x) with all elements beside the diagonal below 2^-5 together, because the fixed point
+// 1/4, not both U and g(x) with elements beside the diagonal below 2^-6 together, because the fixed point
 // truncates them at 2^-60, where FP64 products of such matrices would err by 2^-53 of those elements.
 struct limb_norm {  // squares of the limbs to 12 bits: 2^24 is a length of 1
-  static constexpr unsigned one = 1u << 24, shortest = one / 16, row = 17028874, matrix = 51170508, offdiag = 1u << 14;
+  static constexpr unsigned one = 1u << 24, shortest = one / 16, row = 17028874, matrix = 51170508, offdiag = 1u << 12;
   __device__ static __forceinline__ unsigned of(clq a) {
     const int x = a.r.h >> 18, y = a.i.h >> 18;
     return (unsigned)(x * x + y * y);
