@@ -455,7 +455,7 @@ __device__ __noinline__ void conjugate_average(herm *y, const m3<double> *g) {
 
 // dF/d omega^a(x), a = 0..7, written site-major (V x 8), scaled by `scale` (the incoming gradient). U: the
 // caller's links; g in limb planes and in planes of doubles. The staple is summed in 59 fractional bits (its elements reach 8).
-// Bound by the FP64 pipe (87% busy, 570 of 900 operations in the eleven terms of the series at |omega| = 0.1): 0.64 ms
+// Bound by the FP64 pipe (87% busy, 570 of 900 operations in the eleven terms of the series at |omega| = 0.1): 0.61 ms
 // at 24^4. A step of gradient-based fixing (F, gradient, Fourier filter) took 5.40 ms with Jacobi eigenvectors and FP64
 // products in both calls, and takes 1.57 ms (1.55 without part_check). (The terms below 2^-34 of the sum in float would make it 1.44, with
 // those of links beyond 1e38 infinite.)
